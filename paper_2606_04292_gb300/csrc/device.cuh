@@ -9,6 +9,7 @@
 
 #include <type_traits>
 
+#include "fixlaw.cuh"
 #include "fp64math.cuh"
 
 namespace rich {
@@ -132,90 +133,109 @@ struct Xfer {                    // fine level -> next coarser level
 // Constitutive laws (Table 1 of the paper); psi >= 0 gives theta_s, Ks and a
 // zero capacity for all three laws.
 // ---------------------------------------------------------------------------
-template <int MODEL>
-__device__ __forceinline__ void law_d(double psi, double p1, double p2, const Phys<double>& P,
-                                      double& th, double& dth) {
-  if (!(psi < 0.0)) { th = P.ts; dth = 0.0; return; }
-  const double h = -psi, ds = P.ts - P.tr;
-  if (MODEL == HAVERKAMP) {
-    // theta = theta_r + alpha ds / (alpha + h^beta)
-    const double u = fx::exp(p2 * fx::log(h));
-    const double den = p1 + u;
-    th = P.tr + p1 * ds / den;
-    dth = p1 * ds * p2 * (u / h) / (den * den);
-  } else if (MODEL == GARDNER) {
-    const double e = fx::exp(p1 * psi);
-    th = P.tr + ds * e;
-    dth = p1 * ds * e;
-  } else {
-    // Se = (1 + t)^-m, t = (alpha h)^n, m = 1 - 1/n
-    const double n = p2, m = 1.0 - 1.0 / n;
-    const double t = fx::exp(n * fx::log(p1 * h));
-    const double Se = fx::exp(-m * fx::log1p(t));
-    th = P.tr + ds * Se;
-    dth = ds * m * n * (t / h) * Se / (1.0 + t);
-  }
-}
-
-template <int MODEL>
-__device__ __forceinline__ double theta_only_dm(double psi, double p1, double p2, double m, const Phys<double>& P) {
-  if (!(psi < 0.0)) return P.ts;
-  const double h = -psi, ds = P.ts - P.tr;
-  if (MODEL == HAVERKAMP) return P.tr + p1 * ds / (p1 + fx::exp(p2 * fx::log(h)));
-  if (MODEL == GARDNER) return P.tr + ds * fx::exp(p1 * psi);
-  const double n = p2;
-  return P.tr + ds * fx::exp(-m * fx::log1p(fx::exp(n * fx::log(p1 * h))));
-}
-
-// van Genuchten's m = 1 - 1/n (kernels that evaluate the laws of a per-cell
-// n field read it from a copy made with this same expression)
+// FP64 heads: the powers of a law run in 64-bit fixed point (fixlaw.cuh);
+// arguments outside its ranges take the FP64 functions (slow_*: not inlined,
+// they are all but never reached and would double every kernel's code).
 __device__ __forceinline__ double vg_m(double n) { return 1.0 - 1.0 / n; }
 
-// theta of one law; m (van Genuchten only) from n
+template <int MODEL>
+__device__ __noinline__ double slow_se(double h, double p1, double p2) {
+  if (MODEL == HAVERKAMP) return p1 / (p1 + fx::exp(p2 * fx::log(h)));
+  if (MODEL == GARDNER) return fx::exp(-(p1 * h));
+  return fx::exp(-vg_m(p2) * fx::log1p(fx::exp(p2 * fx::log(p1 * h))));
+}
+
+// Se and d Se/d psi without its factor (Haverkamp beta, Gardner alpha, van
+// Genuchten n - 1)
+template <int MODEL>
+__device__ __noinline__ double2 slow_se_slope(double h, double p1, double p2) {
+  if (MODEL == HAVERKAMP) {
+    const double u = fx::exp(p2 * fx::log(h));
+    const double den = p1 + u;
+    return make_double2(p1 / den, p1 * (u / h) / (den * den));
+  }
+  if (MODEL == GARDNER) {
+    const double e = fx::exp(-(p1 * h));
+    return make_double2(e, e);
+  }
+  const double t = fx::exp(p2 * fx::log(p1 * h));
+  const double Se = fx::exp(-vg_m(p2) * fx::log1p(t));
+  return make_double2(Se, (t / h) * Se / (1.0 + t));
+}
+
+// K/Ks.  For van Genuchten-Mualem, Se^{1/m} = 1/(1+t), so 1 - (1 - Se^{1/m})^m
+// = -expm1(m log(t/(1+t))), evaluated without cancellation in both the wet
+// (t < 1) and the dry (t > 1) range.  With lt = log t and e = exp(-|lt|):
+//   log(1 + t)       = log1p(e) + max(lt, 0),
+//   log(t / (1 + t)) = min(lt, 0) - log1p(e).
+template <int MODEL>
+__device__ __noinline__ double slow_kr(double h, double p1, double p2, double p3, double p4) {
+  if (MODEL == HAVERKAMP) return p3 / (p3 + fx::exp(p4 * fx::log(h)));
+  if (MODEL == GARDNER) return fx::exp(-(p1 * h));
+  const double m = vg_m(p2), lt = p2 * fx::log(p1 * h);
+  const double l1 = fx::log1p(fx::exp(-fabs(lt)));
+  const double inner = -fx::expm1(m * (fmin(lt, 0.0) - l1));
+  return fx::exp(-p3 * m * (l1 + fmax(lt, 0.0))) * inner * inner;
+}
+
+// psi < 0 from its bits (false for +-0 and NaN)
+__device__ __forceinline__ bool unsaturated(double psi) {
+  const unsigned long long b = fl::dbits(psi);
+  return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
+}
+
+// A cell's law with its parameters prepared once per point solve.
+template <int MODEL>
+struct LawCell {
+  fl::Prep q;
+  double p1, p2, ds, cs;      // cs: the factor of d theta/d psi (ds beta, ds alpha, ds (n - 1))
+  __device__ __forceinline__ LawCell(double a, double b, const Phys<double>& P) : p1(a), p2(b), ds(P.ts - P.tr) {
+    if (MODEL != GARDNER) q = fl::prep<MODEL == VANGENUCHTEN>(a, b);
+    cs = ds * (MODEL == GARDNER ? a : (MODEL == HAVERKAMP ? b : b - 1.0));
+  }
+  // theta(psi) and theta'(psi)
+  __device__ __forceinline__ void eval(double psi, const Phys<double>& P, double& th, double& dth) const {
+    if (!unsaturated(psi)) { th = P.ts; dth = 0.0; return; }
+    const unsigned long long hb = fl::dbits(psi) ^ 0x8000000000000000ull;
+    double Se, s;
+    bool ok = true;
+    if (MODEL == GARDNER) {
+      Se = s = fl::exp_gardner(p1, hb, ok);
+    } else {
+      ok = q.ok;
+      fl::se_slope<MODEL == VANGENUCHTEN>(q, hb, ok, Se, s);
+    }
+    if (!ok) {
+      const double2 v = slow_se_slope<MODEL>(-psi, p1, p2);
+      Se = v.x;
+      s = v.y;
+    }
+    th = P.tr + ds * Se;
+    dth = cs * s;
+  }
+};
+
 template <int MODEL>
 __device__ __forceinline__ double theta_only_d(double psi, double p1, double p2, const Phys<double>& P) {
-  return theta_only_dm<MODEL>(psi, p1, p2, (MODEL == VANGENUCHTEN && psi < 0.0) ? vg_m(p2) : 0.0, P);
+  if (!unsaturated(psi)) return P.ts;
+  const unsigned long long hb = fl::dbits(psi) ^ 0x8000000000000000ull;
+  bool ok = true;
+  double Se = MODEL == GARDNER ? fl::exp_gardner(p1, hb, ok) : fl::se_only<MODEL == VANGENUCHTEN>(p1, p2, hb, ok);
+  if (!ok) Se = slow_se<MODEL>(-psi, p1, p2);
+  return P.tr + (P.ts - P.tr) * Se;
 }
 
-// Hydraulic conductivity.  For van Genuchten-Mualem, Se^{1/m} = 1/(1+t), so
-// 1 - (1 - Se^{1/m})^m = -expm1(m log(t/(1+t))), evaluated without
-// cancellation in both the wet (t < 1) and the dry (t > 1) range.  With
-// lt = log t and e = exp(-|lt|) (t when t <= 1, 1/t when t > 1):
-//   log(1 + t)       = log1p(e) + max(lt, 0),
-//   log(t / (1 + t)) = min(lt, 0) - log1p(e),
-// one exponential and one log1p for both ranges, no division and no branch.
-template <int MODEL>
-__device__ __forceinline__ double cond_dm(double psi, double p1, double p2, double m, double Ks,
-                                          const Phys<double>& P) {
-  if (!(psi < 0.0)) return Ks;
-  const double h = -psi;
-  if (MODEL == HAVERKAMP) return Ks * P.p3 / (P.p3 + fx::exp(P.p4 * fx::log(h)));
-  if (MODEL == GARDNER) return Ks * fx::exp(p1 * psi);
-  const double n = p2;
-  const double lt = n * fx::log(p1 * h);
-  const double l1 = fx::log1p(fx::exp(-fabs(lt)));
-  const double L1 = l1 + fmax(lt, 0.0);
-  const double lr = fmin(lt, 0.0) - l1;
-  const double inner = -fx::expm1(m * lr);
-  return Ks * fx::exp(-P.p3 * m * L1) * inner * inner;
-}
-
+// Hydraulic conductivity.
 template <int MODEL>
 __device__ __forceinline__ double cond_d(double psi, double p1, double p2, double Ks, const Phys<double>& P) {
-  return cond_dm<MODEL>(psi, p1, p2, (MODEL == VANGENUCHTEN && psi < 0.0) ? vg_m(p2) : 0.0, Ks, P);
-}
-
-__device__ __forceinline__ double cond_model_d(int model, double psi, double p1, double p2,
-                                               double Ks, const Phys<double>& P) {
-  if (model == HAVERKAMP) return cond_d<HAVERKAMP>(psi, p1, p2, Ks, P);
-  if (model == GARDNER) return cond_d<GARDNER>(psi, p1, p2, Ks, P);
-  return cond_d<VANGENUCHTEN>(psi, p1, p2, Ks, P);
-}
-__device__ __forceinline__ double theta_model_d(int model, double psi, double p1, double p2,
-                                                const Phys<double>& P) {
-  if (model == HAVERKAMP) return theta_only_d<HAVERKAMP>(psi, p1, p2, P);
-  if (model == GARDNER) return theta_only_d<GARDNER>(psi, p1, p2, P);
-  return theta_only_d<VANGENUCHTEN>(psi, p1, p2, P);
+  if (!unsaturated(psi)) return Ks;
+  const unsigned long long hb = fl::dbits(psi) ^ 0x8000000000000000ull;
+  bool ok = true;
+  double Kr = MODEL == HAVERKAMP ? fl::kr_haverkamp(P.p3, P.p4, hb, ok)
+              : MODEL == GARDNER ? fl::exp_gardner(p1, hb, ok)
+                                 : fl::kr_vangenuchten(p1, p2, P.p3, hb, ok);
+  if (!ok) Kr = slow_kr<MODEL>(-psi, p1, p2, P.p3, P.p4);
+  return Ks * Kr;
 }
 
 // Increment form in FP32: Dth = theta(psi0 + x) - theta(psi0) and
@@ -554,26 +574,33 @@ __device__ __forceinline__ double tol_of<double>() { return 1e-15; }
 template <>
 __device__ __forceinline__ float tol_of<float>() { return 1e-7f; }
 
-// Storage + sink part and its derivative at x for either form.
+// Storage + sink part at x for either form (the defect's part of N).
 template <typename T, int FORM, int MODEL>
-__device__ __forceinline__ void storage(T x, T psi0, T p1, T p2, T smax, const Phys<T>& P,
-                                        T& val, T& der) {
+__device__ __forceinline__ T storage(T x, T psi0, T p1, T p2, T smax, const Phys<T>& P) {
   if constexpr (FORM == FORM_DIRECT) {
     static_assert(sizeof(T) == 8, "direct form is FP64");
-    double th, dth, S, dS;
-    law_d<MODEL>(x, p1, p2, P, th, dth);
+    double S, dS;
     sink_direct(x, smax, P, S, dS);
-    val = P.a * th + S;
-    der = P.a * dth + dS;
+    return P.a * theta_only_d<MODEL>(x, p1, p2, P) + S;
   } else {
     static_assert(sizeof(T) == 4, "increment form is FP32");
     float Dth, dth, DS, dS;
     dlaw_fast<MODEL>(psi0, x, p1, p2, P, Dth, dth);
     sink_delta(psi0, x, smax, P, DS, dS);
-    val = P.a * Dth + DS;
-    der = P.a * dth + dS;
+    return P.a * Dth + DS;
   }
 }
+
+// the FP64 law of a point solve (nothing to prepare in the increment form)
+template <int FORM, int MODEL>
+struct PointLaw {
+  template <typename T>
+  __device__ __forceinline__ PointLaw(T, T, const Phys<T>&) {}
+};
+template <int MODEL>
+struct PointLaw<FORM_DIRECT, MODEL> : LawCell<MODEL> {
+  __device__ __forceinline__ PointLaw(double p1, double p2, const Phys<double>& P) : LawCell<MODEL>(p1, p2, P) {}
+};
 
 // Scalar solve of  storage(x) + cc x = f  (eq. point-update).  The left side
 // increases strictly (cc > 0), the root lies in [lo, hi]; Newton from x0,
@@ -612,6 +639,7 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
   }
   T x = x0 < lo ? lo : (x0 > hi ? hi : x0);
   const int maxit = NK > 0 ? NK : (P.newton_k > 0 ? P.newton_k : 200);
+  const PointLaw<FORM, MODEL> law(p1, p2, P);
   DBase B;
   T sa0 = T(0), sda0 = T(0);
   int sk0 = 0;
@@ -637,7 +665,11 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
       val = P.a * Dth + DS;
       der = P.a * dth + dS;
     } else {
-      storage<T, FORM, MODEL>(x, psi0, p1, p2, smax, P, val, der);
+      T th, dth, S, dS;
+      law.eval(x, P, th, dth);
+      sink_direct(x, smax, P, S, dS);
+      val = P.a * th + S;
+      der = P.a * dth + dS;
     }
     const T F = val + cc * x - f;
     const T dF = der + cc;
@@ -776,10 +808,8 @@ __device__ __forceinline__ void cell_sums(const Level<T>& L, const CellOps<T>& c
 // (the expression of apply_N(), so both give the same bits)
 template <typename T, int FORM, int MODEL>
 __device__ __forceinline__ T cell_defect(const Phys<T>& P, const CellOps<T>& c, T dg, T of, T x) {
-  T val, der;
-  with_law<MODEL>(P, c.mat, [&](auto law, const Phys<T>& Q) {
-    storage<T, FORM, decltype(law)::value>(x, c.psi0, c.p1, c.p2, c.smax, Q, val, der);
-    return 0;
+  const T val = with_law<MODEL>(P, c.mat, [&](auto law, const Phys<T>& Q) {
+    return storage<T, FORM, decltype(law)::value>(x, c.psi0, c.p1, c.p2, c.smax, Q);
   });
   return c.g - (val + P.xi * x + dg * x - of);
 }
@@ -811,10 +841,8 @@ __device__ __forceinline__ T apply_N(const Level<T>& L, const Phys<T>& P, const 
   const T p2 = L.p2 ? L.p2[q] : P.p2;
   const T smax = L.smax ? L.smax[q] : T(0);
   const T psi0 = FORM == FORM_DELTA ? L.psi0[q] : T(0);
-  T val, der;
-  with_law<MODEL>(P, mat_of<MODEL>(L, i), [&](auto law, const Phys<T>& Q) {
-    storage<T, FORM, decltype(law)::value>(u[i], psi0, p1, p2, smax, Q, val, der);
-    return 0;
+  const T val = with_law<MODEL>(P, mat_of<MODEL>(L, i), [&](auto law, const Phys<T>& Q) {
+    return storage<T, FORM, decltype(law)::value>(u[i], psi0, p1, p2, smax, Q);
   });
   return val + P.xi * u[i] + mii * u[i] - off;
 }

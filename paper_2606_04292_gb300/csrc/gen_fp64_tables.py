@@ -8,6 +8,11 @@ second double (lo) where a pair is kept:
   log(1 + k/256) (k < 128), log((1 + k/256)/2) (k >= 128) and 1/(1 + k/256)
                                                     (log, log1p)
   ln 2 / 256 and ln 2 split so that a multiple by a small integer is exact.
+The integer tables of the fixed-point laws (fixlaw.cuh) are rounded once to
+the nearest integer of their scale:
+  c_j, the smallest multiple of 1/256 that is at least 64/(64 + j), and
+  -log2 c_j (scale 2^62), j = 0 .. 64; 2^(-k/64) (scale 2^63), k = 0 .. 63;
+  the Taylor coefficients of log2(1 + z)/z and (1 - 2^-r)/r.
 """
 import math
 from decimal import Decimal, getcontext
@@ -60,6 +65,38 @@ for k in range(256):
     a, b = pair((F if k < 128 else F / 2).ln())
     lines.append(f"    {{{hx(a)}, {hx(b)}, {hx(1 / F)}}},")
 lines.append("};")
-lines += ["", "}  // namespace fx", "}  // namespace rich", ""]
+lines += ["", "}  // namespace fx", "", "namespace fl {", ""]
+
+
+def fix(d, bits):
+    return int((d * (1 << bits)).to_integral_value(rounding="ROUND_HALF_EVEN"))
+
+
+lines.append("// 256 c_j and -log2 c_j (scale 2^62), c_j the least multiple of 1/256 >= 64/(64 + j)")
+lines.append("__device__ const unsigned long long kLog2C[65][2] = {")
+zmax = 0
+for j in range(65):
+    C = -(-256 * 64 // (64 + j))
+    lines.append(f"    {{{C}ull, {fix(-(Decimal(C) / 256).ln() / LN2, 62)}ull}},")
+    zmax = max(zmax, (Decimal(65 + j) / 64) * C / 256 - 1) if j < 64 else zmax
+lines.append("};")
+lines.append(f"// (z = c_j M - 1 < {float(zmax):.5f})")
+lines.append("// 2^(-k/64) (scale 2^63)")
+lines.append("__device__ const unsigned long long kExp2N[64] = {")
+for k in range(64):
+    lines.append(f"    {fix((-LN2 * k / 64).exp(), 63)}ull,")
+lines.append("};")
+lines.append("// 1/((k + 1) ln 2): k = 0..4 at scale 2^62, k = 5..10 at scale 2^34")
+for k in range(5):
+    lines.append(f"constexpr unsigned long long LQ{k} = {fix(1 / (LN2 * (k + 1)), 62)}ull;")
+for k in range(5, 11):
+    lines.append(f"constexpr unsigned LQ{k} = {fix(1 / (LN2 * (k + 1)), 34)}u;")
+lines.append("// (ln 2)^(k+1)/(k + 1)!: k = 0..3 at scale 2^64, k = 4..7 at scale 2^41")
+for k in range(4):
+    lines.append(f"constexpr unsigned long long EG{k} = {fix(LN2 ** (k + 1) / math.factorial(k + 1), 64)}ull;")
+for k in range(4, 8):
+    lines.append(f"constexpr unsigned EG{k} = {fix(LN2 ** (k + 1) / math.factorial(k + 1), 41)}u;")
+lines.append(f"constexpr unsigned long long LOG2E_63 = {fix(1 / LN2, 63)}ull;   // log2 e, scale 2^63")
+lines += ["", "}  // namespace fl", "}  // namespace rich", ""]
 with open("fp64_tables.h", "w") as f:
     f.write("\n".join(lines))
