@@ -615,10 +615,27 @@ struct PointLaw<FORM_DIRECT, MODEL> : LawCell<MODEL> {
 // bisect take exactly the fixed count, as before.
 constexpr int BISECT_EXTRA = 12;
 
+// Comparisons of the point solve.  FP64: on the bits, with integers
+// (fixlaw.cuh); an operand that is not a number only has to keep the result
+// one (clamp_to leaves it; a bracket test that fails bisects NaN ends).
+__device__ __forceinline__ bool less(float a, float b) { return a < b; }
+__device__ __forceinline__ bool less(double a, double b) { return fl::order_key(a) < fl::order_key(b); }
+__device__ __forceinline__ bool at_most(float a, float b) { return a <= b; }
+__device__ __forceinline__ bool at_most(double a, double b) { return !less(b, a); }   // (false for a NaN |a|)
+__device__ __forceinline__ bool is_zero(float a) { return a == 0.0f; }
+__device__ __forceinline__ bool is_zero(double a) { return (fl::dbits(a) << 1) == 0; }
+__device__ __forceinline__ bool above_zero(float a) { return a > 0.0f; }
+__device__ __forceinline__ bool above_zero(double a) { return (long long)fl::dbits(a) > 0 && !fl::is_nan(a); }
+__device__ __forceinline__ float clamp_to(float x, float lo, float hi) { return x < lo ? lo : (x > hi ? hi : x); }
+__device__ __forceinline__ double clamp_to(double x, double lo, double hi) {
+  if (fl::is_nan(x) || fl::is_nan(lo) || fl::is_nan(hi)) return x;
+  return less(x, lo) ? lo : (less(hi, x) ? hi : x);
+}
+
 template <typename T, int FORM, int MODEL, int NK = 0>
 __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T smax,
                                          const Phys<T>& P) {
-  if (!(cc > T(0))) {
+  if (!above_zero(cc)) {
     // no coupling and no shift (c = 0): shift kappa (x - x0), kappa = 1e-6 a,
     // which keeps the root and provides the bracket
     const T k = T(1e-6) * P.a;
@@ -628,8 +645,9 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
   const T ds = P.ts - P.tr;
   T lo, hi;
   if constexpr (FORM == FORM_DIRECT) {
-    lo = (f - P.a * P.ts - smax) / cc;
-    hi = (f - P.a * P.tr) / cc;
+    const fl::Divisor dc = fl::divisor(cc);
+    lo = fl::div(f - P.a * P.ts - smax, dc);
+    hi = fl::div(f - P.a * P.tr, dc);
   } else {
     // FP32: both ends through one approximate reciprocal; each end has a
     // slack of (a ds + smax)/cc beyond the root, far above its 2^-22 error
@@ -637,7 +655,7 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
     lo = (f - P.a * ds - smax) * rc;
     hi = (f + P.a * ds + smax) * rc;
   }
-  T x = x0 < lo ? lo : (x0 > hi ? hi : x0);
+  T x = clamp_to(x0, lo, hi);
   const int maxit = NK > 0 ? NK : (P.newton_k > 0 ? P.newton_k : 200);
   const PointLaw<FORM, MODEL> law(p1, p2, P);
   DBase B;
@@ -673,25 +691,26 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
     }
     const T F = val + cc * x - f;
     const T dF = der + cc;
-    if (F == T(0)) return true;
-    if (F > T(0)) hi = x; else lo = x;
+    if (is_zero(F)) return true;
+    if (above_zero(F)) hi = x; else lo = x;
     T xn;
     if constexpr (sizeof(T) == 4) xn = x - __fdividef(F, dF);    // dF > 0; a 2-ulp step error is harmless
-    else xn = x - F / dF;
+    else xn = x - fl::div(F, fl::divisor(dF));
     // a step strictly inside the bracket, or below round-off, is kept;
     // anything else (outside, or onto an end) is replaced by bisection
-    const T tiny = tol_of<T>() * (fabs(x) > T(1) ? fabs(x) : T(1));
-    if (!(xn > lo && xn < hi) && !(fabs(xn - x) <= tiny)) {
+    auto below_roundoff = [&](T s) { return at_most(T(fabs(s)), tol_of<T>() * (less(T(1), fabs(x)) ? fabs(x) : T(1))); };
+    if (!(less(lo, xn) && less(xn, hi)) && !below_roundoff(xn - x)) {
       xn = T(0.5) * (lo + hi);
       *bis = true;
     }
-    const T stp = fabs(xn - x);
+    const T stp = xn - x;
+    const bool last = NK == 0 && P.newton_k <= 0 && below_roundoff(stp);
     x = xn;
-    if (NK == 0 && P.newton_k <= 0 && stp <= tiny) return true;
+    if (last) return true;
     // FP32 increment form: a step below 2^-20 of |x| leaves nothing for the
     // next one to change at this precision (quadratic convergence)
     if constexpr (FORM == FORM_DELTA) {
-      if (stp <= 9.5367431640625e-7f * fabsf(x)) return true;
+      if (fabsf(stp) <= 9.5367431640625e-7f * fabsf(x)) return true;
     }
     return false;
   };

@@ -360,5 +360,48 @@ RICH_FD double exp_gardner(double alpha, u64 hb, bool& ok) {
   return to_double_1(exp2_neg56(e > 5 ? 0 : shr(u, 5 - e)));
 }
 
+// ---------------------------------------------------------------------------
+// FP64 comparisons and quotients off the FP64 pipe (a compare issues there as
+// slowly as an add, a division as eight to ten of them).
+// ---------------------------------------------------------------------------
+// the order of finite and infinite doubles as signed integers (-0 = +0)
+RICH_FD i64 order_key(double x) {
+  const i64 b = (i64)dbits(x);
+  return b < 0 ? (i64)(0x8000000000000000ull - (u64)b) : b;
+}
+RICH_FD bool is_nan(double x) { return (dbits(x) << 1) > 0xffe0000000000000ull; }
+
+// A divisor b and its reciprocal, rounded to nearest from 61 bits (integer
+// Newton-Raphson).  div(a) is Markstein's quotient (IBM J. Res. Dev. 34,
+// 1990): q = a y, then q + (a - b q) y, the correctly rounded a/b.  Exponents
+// near the ends of the range, where a - b q could leave it, divide plainly.
+struct Divisor {
+  double b, y;
+  int e;
+};
+RICH_FD Divisor divisor(double b) {
+  Divisor d;
+  const u64 k = dbits(b);
+  const int e = (int)((k >> 52) & 0x7ff);
+  const u64 r = recip_mant((k << 11) | 0x8000000000000000ull);
+  d.b = b;
+  d.e = e;
+  d.y = bitsd((k & 0x8000000000000000ull) | (((u64)(2044 - e) << 52) + (r >> 11) + ((r >> 10) & 1)));
+  return d;
+}
+// whether div applies: 2^-400 <= |a|, |b| < 2^400, or a = 0
+RICH_FD bool div_ok(double a, const Divisor& d) {
+  const u64 k = dbits(a) << 1;
+  return (u32)(d.e - 623) < 800u && ((u32)((int)(k >> 53) - 623) < 800u || k == 0);
+}
+#ifdef __CUDACC__
+static __device__ __noinline__ double slow_div(double a, double b) { return a / b; }
+RICH_FD double div(double a, const Divisor& d) {
+  if (!div_ok(a, d)) return slow_div(a, d.b);
+  const double q = a * d.y;
+  return fma(fma(-q, d.b, a), d.y, q);
+}
+#endif
+
 }  // namespace fl
 }  // namespace rich
