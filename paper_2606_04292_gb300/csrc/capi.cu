@@ -425,6 +425,7 @@ Level<double> view64(const richards_ctx* c, int l) {
   V.psi0 = nullptr;
   for (int f = 0; f < 6; ++f) V.kb[f] = H.kb[f];
   V.mat = c->layered ? H.mat : nullptr;
+  rich::set_divisors(V);
   return V;
 }
 
@@ -443,6 +444,7 @@ Level<float> view32(const richards_ctx* c, int l) {
   for (int f = 0; f < 6; ++f) V.kb[f] = H.kbf[f];
   V.mat = c->layered ? H.mat : nullptr;
   V.cs = H.cs;
+  rich::set_divisors(V);
   return V;
 }
 

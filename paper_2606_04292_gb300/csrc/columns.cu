@@ -52,96 +52,69 @@ struct ColArgs {
       model;
 };
 
-// The interpolation row of fine cell i (the same reading as the tables of the
-// multi-dimensional path: coarse coordinate ((2i+1) nc - nf)/(2 nf), a ghost
-// beyond an end folded into the end cell with factor slo/shi) in FP32 and
-// 32-bit integers: columns have at most RICHARDS_COLUMN_MAX_CELLS cells.
-__device__ __forceinline__ void interp_row_f(int nf, int nc, int i, float slo, float shi, int* idx, float* w,
-                                             int& cnt) {
-  cnt = 0;
-  auto add = [&](int j, float wt) {
-    if (wt == 0.0f) return;
-    for (int k = 0; k < cnt; ++k)
-      if (idx[k] == j) { w[k] += wt; return; }
-    idx[cnt] = j;
-    w[cnt] = wt;
-    ++cnt;
-  };
-  if (nf == 1) { add(0, 1.0f); return; }
-  const int num = (2 * i + 1) * nc - nf, den = 2 * nf;
-  // floor(num / den) through the FP32 quotient, then corrected: |num| and den
-  // are below 2^24 (exact in FP32) and the quotient's floor is off by at most
-  // one, so one test each way gives the exact integer floor
-  int J0 = (int)floorf(__fdividef((float)num, (float)den));
-  if (J0 * den > num) --J0;
-  else if ((J0 + 1) * den <= num) ++J0;
-  const float wt = (float)(num - J0 * den) / (float)den;
-  const int J1 = J0 + 1;
-  if (J0 < 0) add(0, (1.0f - wt) * slo); else add(J0, 1.0f - wt);
-  if (J1 >= nc) add(nc - 1, wt * shi); else add(J1, wt);
-}
-
 // 1D hierarchy of one column in shared memory; transfer weights computed on
-// the fly (columns have arbitrary lengths) in FP32: R is the transpose of the
-// constant-extrapolation P with rows normalised to 1, P folds the ghost with
-// slo/shi (-1 on a Dirichlet end).
+// the fly (columns have arbitrary lengths, nf -> nc = ceil(nf/2)): the coarse
+// coordinate of fine cell i is num/den = ((2i+1) nc - nf)/(2 nf), so with the
+// integer offset e = num - J den of coarse cell J, its weight is the hat
+// (den - |e|)/den.  R is the transpose of the constant-extrapolation P with
+// rows normalised to 1 (the factor 1/den drops out), P folds the ghost with
+// slo/shi (-1 on a Dirichlet end).  Integers are exact; a row costs ~30
+// instructions, half of the 4096-column step's transfers with the floor
+// divisions of the general interpolation row.
 struct ColumnLevels {
   const Level<float>* Ls;
   float slo, shi;
   __device__ const Level<float>& L(int l) const { return Ls[l]; }
-  // the taps of coarse row J0: fine indices ri, weights rw (cnt of them) and
-  // the inverse of their sum
-  __device__ int taps(int l, int J0, int* ri, float* rw, float& inv) const {
-    const int nf = Ls[l].n0, nc = Ls[l + 1].n0;
-    int cnt = 0;
-    // (nc = ceil(nf/2): a fine cell i reaches coarse rows floor(t), floor(t) + 1
-    // with t = ((2i+1) nc - nf) / (2 nf), so the cells of row J0 lie in
-    // [2 J0 - 2, 2 J0 + 2]; checked for every nf up to 2048)
-    const int lo = nf == 1 ? 0 : max(0, 2 * J0 - 2), hi = nf == 1 ? 0 : min(nf - 1, 2 * J0 + 2);
-    for (int i = lo; i <= hi; ++i) {
-      int idx[2];
-      float w[2];
-      int c2;
-      interp_row_f(nf, nc, i, 1.0f, 1.0f, idx, w, c2);
-      for (int k = 0; k < c2; ++k)
-        if (idx[k] == J0 && cnt < RMAX) { ri[cnt] = i; rw[cnt] = w[k]; ++cnt; }
+  // weights (integers) of the fine cells 2 J - 2 .. 2 J + 2, the only ones
+  // that reach coarse row J, and the inverse of their sum
+  __device__ __forceinline__ float taps(int l, int J, float* w) const {
+    const int nf = Ls[l].n0, nc = Ls[l + 1].n0, den = 2 * nf;
+    int s = 0, e = (4 * J - 3) * nc - nf - J * den;
+#pragma unroll
+    for (int k = 0; k < 5; ++k, e += 2 * nc) {
+      const int i = 2 * J - 2 + k;
+      int d = e;                        // beyond an end the weight stays 1
+      if (J == 0) d = max(d, 0);
+      if (J == nc - 1) d = min(d, 0);
+      const int wi = (i >= 0 && i < nf) ? max(den - abs(d), 0) : 0;
+      s += wi;
+      w[k] = (float)wi;
     }
-    float s = 0.0f;
-    for (int k = 0; k < cnt; ++k) s += rw[k];
-    inv = 1.0f / s;
-    return cnt;
+    return 1.0f / (float)s;
   }
-  __device__ float restrict(int l, const float* fine, int J0, int, int) const {
-    int ri[RMAX];
-    float rw[RMAX], inv;
-    const int cnt = taps(l, J0, ri, rw, inv);
+  __device__ float restrict(int l, const float* fine, int J, int, int) const {
+    float w[5];
+    const float inv = taps(l, J, w);
     float acc = 0.0f;
-    for (int k = 0; k < cnt; ++k) acc += rw[k] * inv * fine[ri[k]];
+#pragma unroll
+    for (int k = 0; k < 5; ++k)
+      if (w[k] != 0.0f) acc += w[k] * inv * fine[2 * J - 2 + k];
     return acc;
   }
-  // two arrays through one computation of the taps (the same sums as two
-  // restrict calls)
-  __device__ void restrict2(int l, const float* fa, const float* fb, int J0, int, int, float& a, float& b) const {
-    int ri[RMAX];
-    float rw[RMAX], inv;
-    const int cnt = taps(l, J0, ri, rw, inv);
+  // two arrays through one computation of the taps
+  __device__ void restrict2(int l, const float* fa, const float* fb, int J, int, int, float& a, float& b) const {
+    float w[5];
+    const float inv = taps(l, J, w);
     float sa = 0.0f, sb = 0.0f;
-    for (int k = 0; k < cnt; ++k) {
-      sa += rw[k] * inv * fa[ri[k]];
-      sb += rw[k] * inv * fb[ri[k]];
-    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k)
+      if (w[k] != 0.0f) {
+        sa += w[k] * inv * fa[2 * J - 2 + k];
+        sb += w[k] * inv * fb[2 * J - 2 + k];
+      }
     a = sa;
     b = sb;
   }
-  __device__ float prolong(int l, int i0, int, int) const {
+  __device__ float prolong(int l, int i, int, int) const {
     const Level<float>& C = Ls[l + 1];
-    int idx[2];
-    float w[2];
-    int cnt;
-    interp_row_f(Ls[l].n0, C.n0, i0, slo, shi, idx, w, cnt);
-    float acc = 0.0f;
-    for (int k = 0; k < cnt; ++k) acc += w[k] * (C.u[idx[k]] - C.ubar[idx[k]]);
-    return acc;
+    const int nf = Ls[l].n0, nc = C.n0, den = 2 * nf;
+    // floor(num/den) is (i - 1) >> 1 or the next integer
+    int J = (i - 1) >> 1, e = (2 * i + 1) * nc - nf - J * den;
+    if (e >= den) { ++J; e -= den; }
+    const float w = (float)e / (float)den;
+    const int a = max(J, 0), b = min(J + 1, nc - 1);
+    const float wa = J < 0 ? (1.0f - w) * slo : 1.0f - w, wb = J + 1 >= nc ? w * shi : w;
+    return wa * (C.u[a] - C.ubar[a]) + wb * (C.u[b] - C.ubar[b]);
   }
 };
 
@@ -165,6 +138,7 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
       V.Kc = p + 4 * nn; V.psi0 = p + 5 * nn; V.smax = A.sink ? p + 6 * nn : nullptr;
       V.p1 = nullptr; V.p2 = nullptr;
       V.mat = nullptr; V.cs = 0;
+      set_divisors(V);
       p += COL_ARRAYS * nn;
       V.kb[0] = p; V.kb[1] = p + 1;
       V.kb[2] = V.kb[3] = V.kb[4] = V.kb[5] = nullptr;

@@ -39,7 +39,26 @@ struct Level {
   const T *kb[6];                // boundary face conductances (per face cell)
   const uint8_t *mat;            // COMPOSITE: material of each cell of this level
   int cs;                        // 1: g, psi0, p1, p2, smax in the colour-split layout (pix)
+  unsigned rn0, rnh, rn1;        // quick_div factors of n0, ceil(n0/2), n1 (set_divisors)
 };
+
+// t / n for the block loops of the small levels (an integer division is ~20
+// dependent instructions, and a phase of the coarse tail does four of them
+// per cell): the high word of t ceil(2^32/n) is exact for t n < 2^32.  Factor
+// 0: n = 1, or a level too big for it (more than 2^16 cells), which divides.
+__host__ __device__ __forceinline__ unsigned div_factor(unsigned n, long long ncell) {
+  return n > 1 && ncell <= 65536 ? 0xffffffffu / n + 1 : 0u;
+}
+__device__ __forceinline__ unsigned quick_div(unsigned t, unsigned n, unsigned factor) {
+  if (factor) return __umulhi(t, factor);
+  return n == 1 ? t : t / n;
+}
+template <typename T>
+__host__ __device__ __forceinline__ void set_divisors(Level<T>& L) {
+  L.rn0 = div_factor((unsigned)L.n0, L.ncell);
+  L.rnh = div_factor((unsigned)((L.n0 + 1) >> 1), L.ncell);
+  L.rn1 = div_factor((unsigned)L.n1, L.ncell);
+}
 
 // Index of cell (i0, i1, i2) (flat index i) in the per-cell parameter arrays
 // g, psi0, p1, p2, smax of a level.  Natural layout: i.  Colour-split layout
@@ -238,103 +257,47 @@ __device__ __forceinline__ double cond_d(double psi, double p1, double p2, doubl
   return Ks * Kr;
 }
 
-// Increment form in FP32: Dth = theta(psi0 + x) - theta(psi0) and
-// dth = theta'(psi0 + x), with the differences taken through expm1/log1p of
-// the ratio (psi0 + x)/psi0, so that Dth is accurate relative to itself.
-template <int MODEL>
-__device__ __forceinline__ void dlaw_f(float psi0, float x, float p1, float p2, const Phys<float>& P,
-                                       float& Dth, float& dth) {
-  const float ds = P.ts - P.tr;
-  const float psi1 = psi0 + x;
-  const bool wet0 = !(psi0 < 0.0f), wet1 = !(psi1 < 0.0f);
-  if (MODEL == GARDNER) {
-    const float al = p1;
-    if (!wet0) {
-      const float e0 = expf(al * psi0);
-      if (!wet1) {
-        const float em = expm1f(al * x);
-        Dth = ds * e0 * em;
-        dth = al * ds * e0 * (1.0f + em);
-      } else {
-        Dth = -ds * expm1f(al * psi0);
-        dth = 0.0f;
-      }
-    } else if (!wet1) {
-      Dth = ds * expm1f(al * psi1);
-      dth = al * ds * expf(al * psi1);
-    } else {
-      Dth = 0.0f; dth = 0.0f;
-    }
-  } else if (MODEL == HAVERKAMP) {
-    const float al = p1, be = p2;
-    if (!wet0) {
-      const float h0 = -psi0;
-      const float u0 = expf(be * logf(h0));
-      if (!wet1) {
-        const float du = u0 * expm1f(be * log1pf(x / psi0));
-        const float u1 = u0 + du, h1 = -psi1;
-        const float den1 = al + u1;
-        Dth = -al * ds * du / ((al + u0) * den1);
-        dth = al * ds * be * (u1 / h1) / (den1 * den1);
-      } else {
-        Dth = ds * u0 / (al + u0);
-        dth = 0.0f;
-      }
-    } else if (!wet1) {
-      const float h1 = -psi1;
-      const float u1 = expf(be * logf(h1));
-      const float den1 = al + u1;
-      Dth = -ds * u1 / den1;
-      dth = al * ds * be * (u1 / h1) / (den1 * den1);
-    } else {
-      Dth = 0.0f; dth = 0.0f;
-    }
-  } else {
-    const float al = p1, n = p2, m = 1.0f - 1.0f / n;
-    if (!wet0) {
-      const float h0 = -psi0;
-      const float t0 = expf(n * logf(al * h0));
-      const float L0 = log1pf(t0);
-      const float Se0 = expf(-m * L0);
-      if (!wet1) {
-        const float dt = t0 * expm1f(n * log1pf(x / psi0));      // t1 - t0
-        const float t1 = t0 + dt;
-        const float dL = log1pf(dt / (1.0f + t0));                // log(1+t1) - log(1+t0)
-        const float dSe = Se0 * expm1f(-m * dL);
-        const float Se1 = Se0 + dSe;
-        Dth = ds * dSe;
-        dth = ds * m * n * (t1 / (-psi1)) * Se1 / (1.0f + t1);
-      } else {
-        Dth = -ds * expm1f(-m * L0);
-        dth = 0.0f;
-      }
-    } else if (!wet1) {
-      const float h1 = -psi1;
-      const float t1 = expf(n * logf(al * h1));
-      const float L1 = log1pf(t1);
-      Dth = ds * expm1f(-m * L1);
-      dth = ds * m * n * (t1 / h1) * expf(-m * L1) / (1.0f + t1);
-    } else {
-      Dth = 0.0f; dth = 0.0f;
-    }
-  }
+// ---------------------------------------------------------------------------
+// Increment form in FP32 for the inner correction problem: Dth =
+// theta(psi0 + x) - theta(psi0) and dth = theta'(psi0 + x), the differences
+// through expm1/log1p of the ratio (psi0 + x)/psi0, so that Dth is accurate
+// relative to itself.  The inner FP32 solve only has to be accurate to ~1e-5
+// relative (the outer defect correction removes the rest), but the increments
+// must stay free of cancellation: log1p and expm1 of small arguments come
+// from their Taylor series (truncation below 1e-10 relative for |x| < 1/32),
+// larger arguments use the hardware approximations (relative error ~1e-6 of
+// a result that is then not small).
+//
+// The hardware's 1/x, log2 and 2^x are taken in their flush-to-zero forms:
+// the plain __fdividef, __logf, __expf wrap each in three to five
+// instructions that rescale subnormal operands, which no operand here needs
+// (a power below 1e-38 adds nothing to 1 + t), and a point update takes 16 of
+// them.  Reciprocals of per-cell values (1/(1 + t0)) are taken once per update.
+// The point update is bound by instruction issue on big levels and by its own
+// instruction chain (~6 cycles per instruction of a lone warp) on small ones.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float rcp_a(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float log_a(float x) {
+  float r;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r * 0.69314718f;
+}
+__device__ __forceinline__ float exp_a(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * 1.44269504f));
+  return r;
 }
 
-// ---------------------------------------------------------------------------
-// Fast single-precision pieces for the inner correction problem.  The inner
-// FP32 solve only has to be accurate to ~1e-5 relative (the float-float outer
-// defect correction removes the rest), but the increments must stay free of
-// cancellation: log1p and expm1 of small arguments come from their Taylor
-// series (truncation below 1e-10 relative for |x| < 1/32), larger arguments
-// use the hardware approximations __logf / __expf (relative error ~1e-6 of a
-// result that is then not small).
-// ---------------------------------------------------------------------------
 // (both forms are evaluated and one is selected: no branch, so lanes of a
 // warp on either side of 1/32 do not split it into two passes)
 __device__ __forceinline__ float fast_log1p(float x) {
   // x - x^2/2 + x^3/3 - x^4/4 + x^5/5 - x^6/6
   const float p = fmaf(x, fmaf(x, fmaf(x, fmaf(x, fmaf(x, -1.0f / 6.0f, 0.2f), -0.25f), 1.0f / 3.0f), -0.5f), 1.0f);
-  const float big = __logf(1.0f + x);
+  const float big = log_a(1.0f + x);
   return fabsf(x) < 0.03125f ? x * p : big;
 }
 
@@ -342,17 +305,18 @@ __device__ __forceinline__ float fast_expm1(float x) {
   // x + x^2/2 + x^3/6 + x^4/24 + x^5/120 + x^6/720
   const float p = fmaf(x, fmaf(x, fmaf(x, fmaf(x, fmaf(x, 1.0f / 720.0f, 1.0f / 120.0f), 1.0f / 24.0f),
                                            1.0f / 6.0f), 0.5f), 1.0f);
-  const float big = __expf(x) - 1.0f;
+  const float big = exp_a(x) - 1.0f;
   return fabsf(x) < 0.03125f ? x * p : big;
 }
 
-// Same increments as dlaw_f, built from the fast pieces above, split into
-// the part that depends on psi0 only (once per point update) and the part
-// that depends on the correction x (once per Newton step).
+// The increment law split into the part that depends on psi0 only (once per
+// point update) and the part that depends on the correction x (once per
+// Newton step).
 struct DBase {
   float psi0, inv_psi0;
   bool wet0;
   float a0, b0, c0;      // VG: t0, log1p(t0), Se0; Haverkamp: u0, log(u0); Gardner: e0
+  float r0;              // VG: 1/(1 + t0); Haverkamp: 1/(alpha + u0)
   float m;               // VG: 1 - 1/n
 };
 
@@ -369,21 +333,23 @@ __device__ __forceinline__ DBase dbase(float psi0, float p1, float p2) {
   DBase B;
   B.psi0 = psi0;
   B.wet0 = !(psi0 < 0.0f);
-  B.inv_psi0 = B.wet0 ? 0.0f : __fdividef(1.0f, psi0);
-  B.a0 = B.b0 = B.c0 = 0.0f;
-  B.m = MODEL == VANGENUCHTEN ? 1.0f - __fdividef(1.0f, p2) : 0.0f;
+  B.inv_psi0 = B.wet0 ? 0.0f : rcp_a(psi0);
+  B.a0 = B.b0 = B.c0 = B.r0 = 0.0f;
+  B.m = MODEL == VANGENUCHTEN ? 1.0f - rcp_a(p2) : 0.0f;
   if (!B.wet0) {
     if (MODEL == GARDNER) {
-      B.a0 = __expf(p1 * psi0);
+      B.a0 = exp_a(p1 * psi0);
     } else if (MODEL == HAVERKAMP) {
-      const float lu = fminf(p2 * __logf(-psi0), POW_EXP_MAX);   // h0^beta through the hardware log/exp
-      B.a0 = __expf(lu);
+      const float lu = fminf(p2 * log_a(-psi0), POW_EXP_MAX);   // h0^beta
+      B.a0 = exp_a(lu);
       B.b0 = lu;
+      B.r0 = rcp_a(p1 + B.a0);
     } else {
       const float m = B.m;
-      B.a0 = __expf(fminf(p2 * __logf(p1 * -psi0), POW_EXP_MAX));   // (alpha h0)^n
+      B.a0 = exp_a(fminf(p2 * log_a(p1 * -psi0), POW_EXP_MAX));   // (alpha h0)^n
       B.b0 = fast_log1p(B.a0);
-      B.c0 = __expf(-m * B.b0);
+      B.c0 = exp_a(-m * B.b0);
+      B.r0 = rcp_a(1.0f + B.a0);
     }
   }
   return B;
@@ -409,7 +375,7 @@ __device__ __forceinline__ void dincr(const DBase& B, float x, float p1, float p
       }
     } else if (!wet1) {
       Dth = ds * fast_expm1(al * psi1);
-      dth = al * ds * __expf(al * psi1);
+      dth = al * ds * exp_a(al * psi1);
     } else {
       Dth = 0.0f; dth = 0.0f;
     }
@@ -422,20 +388,20 @@ __device__ __forceinline__ void dincr(const DBase& B, float x, float p1, float p
         // (psi1/psi0 > 0 here; its rounded value is kept above 2^-24)
         const float q = fmaxf(x * B.inv_psi0, -0.99999994f);
         const float du = u0 * fast_expm1(fminf(be * fast_log1p(q), POW_EXP_MAX - B.b0));
-        const float u1 = u0 + du, h1 = -psi1;
-        const float den1 = al + u1;
-        Dth = __fdividef(-al * ds * du, (al + u0) * den1);
-        dth = __fdividef(al * ds * be * __fdividef(u1, h1), den1 * den1);
+        const float u1 = u0 + du;
+        const float r1 = rcp_a(al + u1);
+        Dth = -al * ds * (du * B.r0) * r1;
+        dth = al * ds * be * (u1 * r1) * (r1 * rcp_a(-psi1));
       } else {
-        Dth = __fdividef(ds * u0, al + u0);
+        Dth = ds * u0 * B.r0;
         dth = 0.0f;
       }
     } else if (!wet1) {
       const float h1 = -psi1;
-      const float u1 = __expf(fminf(be * __logf(h1), POW_EXP_MAX));
-      const float den1 = al + u1;
-      Dth = __fdividef(-ds * u1, den1);
-      dth = __fdividef(al * ds * be * __fdividef(u1, h1), den1 * den1);
+      const float u1 = exp_a(fminf(be * log_a(h1), POW_EXP_MAX));
+      const float r1 = rcp_a(al + u1);
+      Dth = -ds * u1 * r1;
+      dth = al * ds * be * (u1 * r1) * (r1 * rcp_a(h1));
     } else {
       Dth = 0.0f; dth = 0.0f;
     }
@@ -448,20 +414,20 @@ __device__ __forceinline__ void dincr(const DBase& B, float x, float p1, float p
         const float q = fmaxf(x * B.inv_psi0, -0.99999994f);     // (as for Haverkamp)
         const float dt = t0 * fast_expm1(fminf(n * fast_log1p(q), POW_EXP_MAX - B.b0));
         const float t1 = t0 + dt;
-        const float dSe = Se0 * fast_expm1(-m * fast_log1p(__fdividef(dt, 1.0f + t0)));
+        const float dSe = Se0 * fast_expm1(-m * fast_log1p(dt * B.r0));
         const float Se1 = Se0 + dSe;
         Dth = ds * dSe;
-        dth = ds * m * n * __fdividef(t1, -psi1) * __fdividef(Se1, 1.0f + t1);
+        dth = ds * m * n * (t1 * rcp_a(-psi1)) * (Se1 * rcp_a(1.0f + t1));
       } else {
         Dth = -ds * fast_expm1(-m * L0);
         dth = 0.0f;
       }
     } else if (!wet1) {
       const float h1 = -psi1;
-      const float t1 = __expf(fminf(n * __logf(al * h1), POW_EXP_MAX));
+      const float t1 = exp_a(fminf(n * log_a(al * h1), POW_EXP_MAX));
       const float L1 = fast_log1p(t1);
       Dth = ds * fast_expm1(-m * L1);
-      dth = ds * m * n * __fdividef(t1, h1) * __fdividef(__expf(-m * L1), 1.0f + t1);
+      dth = ds * m * n * (t1 * rcp_a(h1)) * (exp_a(-m * L1) * rcp_a(1.0f + t1));
     } else {
       Dth = 0.0f; dth = 0.0f;
     }
@@ -651,7 +617,7 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
   } else {
     // FP32: both ends through one approximate reciprocal; each end has a
     // slack of (a ds + smax)/cc beyond the root, far above its 2^-22 error
-    const T rc = __fdividef(1.0f, cc);
+    const T rc = rcp_a(cc);
     lo = (f - P.a * ds - smax) * rc;
     hi = (f + P.a * ds + smax) * rc;
   }
@@ -694,7 +660,7 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
     if (is_zero(F)) return true;
     if (above_zero(F)) hi = x; else lo = x;
     T xn;
-    if constexpr (sizeof(T) == 4) xn = x - __fdividef(F, dF);    // dF > 0; a 2-ulp step error is harmless
+    if constexpr (sizeof(T) == 4) xn = x - F * rcp_a(dF);        // dF > 0; a 2-ulp step error is harmless
     else xn = x - fl::div(F, fl::divisor(dF));
     // a step strictly inside the bracket, or below round-off, is kept;
     // anything else (outside, or onto an end) is replaced by bisection
@@ -876,18 +842,29 @@ __device__ __forceinline__ void cell_coords(const int n0, const int n1, long lon
   i2 = (int)(r / (unsigned)n1);
 }
 
+// the same through the level's divisor factors
+template <typename T>
+__device__ __forceinline__ void cell_coords(const Level<T>& L, unsigned i, int& i0, int& i1, int& i2) {
+  const unsigned r = quick_div(i, (unsigned)L.n0, L.rn0);
+  const unsigned z = quick_div(r, (unsigned)L.n1, L.rn1);
+  i0 = (int)(i - r * (unsigned)L.n0);
+  i1 = (int)(r - z * (unsigned)L.n1);
+  i2 = (int)z;
+}
+
 // thread index t over one colour -> cell (x pairs, colour chosen per row)
-__device__ __forceinline__ bool color_cell(int n0, int n1, long long t, int color, int& i0, int& i1,
-                                           int& i2, long long& i) {
-  const unsigned nh = (unsigned)((n0 + 1) >> 1);
-  const unsigned ut = (unsigned)t;
-  const unsigned r = ut / nh;
-  const int p = (int)(ut - r * nh);
-  i1 = (int)(r % (unsigned)n1);
-  i2 = (int)(r / (unsigned)n1);
+template <typename T>
+__device__ __forceinline__ bool color_cell(const Level<T>& L, unsigned t, int color, int& i0, int& i1, int& i2,
+                                           unsigned& i) {
+  const unsigned nh = (unsigned)((L.n0 + 1) >> 1);
+  const unsigned r = quick_div(t, nh, L.rnh);
+  const unsigned z = quick_div(r, (unsigned)L.n1, L.rn1);
+  const int p = (int)(t - r * nh);
+  i1 = (int)(r - z * (unsigned)L.n1);
+  i2 = (int)z;
   i0 = 2 * p + ((color + i1 + i2) & 1);
-  if (i0 >= n0) return false;
-  i = i0 + (long long)n0 * (i1 + (long long)n1 * i2);
+  if (i0 >= L.n0) return false;
+  i = (unsigned)i0 + (unsigned)L.n0 * r;
   return true;
 }
 

@@ -534,7 +534,7 @@ __device__ __forceinline__ void block_sweep(const Level<T>& L, const Phys<T>& P,
     const int nrows = L.n1 * L.n2;
     for (int s = 0; s < nplanes; ++s) {
       for (int t = tm.rank(); t < nrows; t += tm.size()) {
-        const int i1 = t % L.n1, i2 = t / L.n1;
+        const int i2 = (int)quick_div((unsigned)t, (unsigned)L.n1, L.rn1), i1 = t - i2 * L.n1;
         const int i0 = s - i1 - i2;
         if (i0 >= 0 && i0 < L.n0)
           point_update<T, FORM, MODEL>(L, P, (unsigned)(i0 + L.n0 * t), i0, i1, i2);
@@ -543,12 +543,12 @@ __device__ __forceinline__ void block_sweep(const Level<T>& L, const Phys<T>& P,
     }
     return;
   }
-  const long long nh = (long long)((L.n0 + 1) >> 1) * L.n1 * L.n2;
+  const unsigned nh = (unsigned)((L.n0 + 1) >> 1) * (unsigned)L.n1 * (unsigned)L.n2;
   for (int color = 0; color < 2; ++color) {
-    for (long long t = tm.rank(); t < nh; t += tm.size()) {
+    for (unsigned t = tm.rank(); t < nh; t += tm.size()) {
       int i0, i1, i2;
-      long long i;
-      if (color_cell(L.n0, L.n1, t, color, i0, i1, i2, i)) point_update<T, FORM, MODEL>(L, P, i, i0, i1, i2);
+      unsigned i;
+      if (color_cell(L, t, color, i0, i1, i2, i)) point_update<T, FORM, MODEL>(L, P, i, i0, i1, i2);
     }
     tm.sync();
   }
@@ -562,7 +562,7 @@ __device__ __forceinline__ T block_defect_norm(const Level<T>& L, const Phys<T>&
   unsigned long long mx = 0;
   for (long long i = tm.rank(); i < L.ncell; i += tm.size()) {
     int i0, i1, i2;
-    cell_coords(L.n0, L.n1, i, i0, i1, i2);
+    cell_coords(L, (unsigned)i, i0, i1, i2);
     const T di = L.g[pix(L, i, i0, i1, i2)] - apply_N<T, FORM, MODEL>(L, P, L.u, i, i0, i1, i2);
     const unsigned long long b = nbits(di);
     mx = b > mx ? b : mx;
@@ -623,20 +623,20 @@ __device__ __forceinline__ void block_cycle(const LV& lv, int l0, int nl, const 
       updates += (unsigned long long)nu1 * F.ncell;
       for (long long i = tm.rank(); i < F.ncell; i += tm.size()) {
         int i0, i1, i2;
-        cell_coords(F.n0, F.n1, i, i0, i1, i2);
+        cell_coords(F, (unsigned)i, i0, i1, i2);
         F.d[i] = F.g[pix(F, i, i0, i1, i2)] - apply_N<T, FORM, MODEL>(F, P, F.u, i, i0, i1, i2);
       }
       tm.sync();
       const Level<T>& C = lv.L(l + 1);
       for (long long J = tm.rank(); J < C.ncell; J += tm.size()) {
         int J0, J1, J2;
-        cell_coords(C.n0, C.n1, J, J0, J1, J2);
+        cell_coords(C, (unsigned)J, J0, J1, J2);
         lv.restrict2(l, F.u, F.d, J0, J1, J2, C.ubar[J], C.d[J]);
       }
       tm.sync();
       for (long long J = tm.rank(); J < C.ncell; J += tm.size()) {
         int J0, J1, J2;
-        cell_coords(C.n0, C.n1, J, J0, J1, J2);
+        cell_coords(C, (unsigned)J, J0, J1, J2);
         C.g[J] = apply_N<T, FORM, MODEL>(C, P, C.ubar, J, J0, J1, J2) + C.d[J];
         C.u[J] = C.ubar[J];
       }
@@ -657,7 +657,7 @@ __device__ __forceinline__ void block_cycle(const LV& lv, int l0, int nl, const 
     const Level<T>& F = lv.L(pl);
     for (long long i = tm.rank(); i < F.ncell; i += tm.size()) {
       int i0, i1, i2;
-      cell_coords(F.n0, F.n1, i, i0, i1, i2);
+      cell_coords(F, (unsigned)i, i0, i1, i2);
       F.u[i] += lv.prolong(pl, i0, i1, i2);
     }
     tm.sync();

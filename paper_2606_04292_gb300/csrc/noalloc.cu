@@ -333,6 +333,7 @@ long long build_plan(const richards_grid* grid, const richards_soil* soil, const
     L.dim = grid->dim;
     L.n0 = n[l][0]; L.n1 = n[l][1]; L.n2 = n[l][2];
     L.ncell = (long long)L.n0 * L.n1 * L.n2;
+    set_divisors(L);
     for (int a = 0; a < 3; ++a) {
       const double h = a < grid->dim ? grid->L[a] / n[l][a] : 1.0;
       L.ih2[a] = a < grid->dim ? 1.0 / (h * h) : 0.0;
