@@ -67,33 +67,32 @@ __global__ void __launch_bounds__(BATCH_THREADS) k_batch32(const BJob32* __restr
   }
 }
 
+// the coarse tail of each listed descriptor by a cluster of blocks of its own
 __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail_batch32(const BJob32* __restrict__ table,
                                                                  const __grid_constant__ BList list, int nu1,
                                                                  int nu2, int cmax, float crtol, int gamma,
                                                                  int gamma_levels) {
-  __shared__ unsigned long long sm[33];
-  const BJob32& J = table[list.job[blockIdx.x]];
+  __shared__ ClusterShared sh;
+  __shared__ Level<float> sL[TEAM_LEVELS];
+  __shared__ Xfer<float> sX[TEAM_LEVELS];
+  ClusterTeam tm(&sh);
+  const BJob32& J = table[list.job[blockIdx.x / tm.nct]];
+  stage_levels(J.dLs, J.dXs, J.level, J.nlev, sL, sX);
+  tm.sync();
   unsigned long long updates = 0;
-  const DeviceLevels<float> lv{J.dLs, J.dXs};
+  const GridLevels<float> lv{sL, sX, J.level, J.tail_start};
+  auto cycle = [&](auto m) {
+    team_cycle<float, FORM_DELTA, decltype(m)::value>(lv, J.level, J.nlev, J.P, nu1, nu2, cmax, crtol, gamma,
+                                                      gamma_levels, updates, 1, J.handoff, tm);
+  };
   switch (J.model) {
-    case HAVERKAMP:
-      block_cycle<float, FORM_DELTA, HAVERKAMP>(lv, J.level, J.nlev, J.P, nu1, nu2, cmax, crtol, gamma,
-                                                gamma_levels, sm, updates, 1);
-      break;
-    case GARDNER:
-      block_cycle<float, FORM_DELTA, GARDNER>(lv, J.level, J.nlev, J.P, nu1, nu2, cmax, crtol, gamma,
-                                              gamma_levels, sm, updates, 1);
-      break;
-    case COMPOSITE:
-      block_cycle<float, FORM_DELTA, COMPOSITE>(lv, J.level, J.nlev, J.P, nu1, nu2, cmax, crtol, gamma,
-                                                gamma_levels, sm, updates, 1);
-      break;
-    default:
-      block_cycle<float, FORM_DELTA, VANGENUCHTEN>(lv, J.level, J.nlev, J.P, nu1, nu2, cmax, crtol, gamma,
-                                                   gamma_levels, sm, updates, 1);
-      break;
+    case HAVERKAMP: cycle(LawTag<HAVERKAMP>{}); break;
+    case GARDNER: cycle(LawTag<GARDNER>{}); break;
+    case COMPOSITE: cycle(LawTag<COMPOSITE>{}); break;
+    default: cycle(LawTag<VANGENUCHTEN>{}); break;
   }
-  if (threadIdx.x == 0 && J.stats) atomicAdd(J.stats, updates);
+  if (threadIdx.x == 0 && tm.lead() && J.stats) atomicAdd(J.stats, updates);
+  tm.sync();
 }
 
 template <int OP, int NK>
@@ -128,10 +127,11 @@ void batch32(int op, int nk, const BJob32* table, const BList& list, int color, 
   }
 }
 
-void batch_tail32(const BJob32* table, const BList& list, int nu1, int nu2, int cmax, float crtol, int gamma,
+void batch_tail32(const BJob32* table, const BList& list, int blocks, int nu1, int nu2, int cmax, float crtol, int gamma,
                   int gamma_levels, cudaStream_t s) {
   if (list.n <= 0) return;
-  k_tail_batch32<<<list.n, TAIL_THREADS, 0, s>>>(table, list, nu1, nu2, cmax, crtol, gamma, gamma_levels);
+  launch_cluster(k_tail_batch32, blocks, list.n, TAIL_THREADS, s, table, list, nu1, nu2, cmax, crtol, gamma,
+                 gamma_levels);
 }
 
 }  // namespace rich

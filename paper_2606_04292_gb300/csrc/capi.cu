@@ -80,6 +80,9 @@ struct richards_ctx {
   richards_grid grid{};
   richards_opts opts{};
   int nlev = 0, tail_start = 0;
+  // first level a cycle runs in the tail's cluster (FP64, FP32, FP32 under a
+  // batcher): at most tail_start
+  int team_start64 = 0, team_start32 = 0, team_start_batch = 0;
   HLevel L[MAXLEV];
   richards_soil soil{};
   bool soil_set = false, het_p1 = false, het_p2 = false, het_Ks = false;
@@ -603,6 +606,26 @@ void smooth32(richards_ctx* c, const Level<float>& F, const Phys<float>& P, int 
   c->updates_host += (long long)nu * F.ncell;
 }
 
+// how the tail from level l runs
+template <typename T>
+rich::TeamShape tail_shape(const richards_ctx* c, int l) {
+  long long cells[MAXLEV];
+  for (int k = 0; k < c->nlev; ++k) cells[k] = c->L[k].ncell;
+  return rich::team_shape<T>(cells, l, c->nlev, c->tail_start);
+}
+
+// first level a cycle runs in the tail's cluster: the coarse tail's, or an
+// earlier one below the finest that is small enough (red-black sweeps: a
+// lexicographic sweep of more cells than the tail's keeps its launches)
+template <typename T>
+int team_start(const richards_ctx* c, bool batched = false) {
+  if (c->opts.ordering != 1) return c->tail_start;
+  for (int l = 1; l < c->tail_start; ++l)
+    if ((long long)c->L[l].n[0] * c->L[l].n[1] * c->L[l].n[2] <= rich::cluster_cells<T>(c->grid.dim, batched))
+      return l;
+  return c->tail_start;
+}
+
 // ------------------------------------------------------------------------
 // One V-cycle (Section 3.2, steps 1-7 with the coarse solve replaced by the
 // recursion) from level l: grid kernels down to the coarse tail, which runs
@@ -612,10 +635,10 @@ void smooth32(richards_ctx* c, const Level<float>& F, const Phys<float>& P, int 
 void vcycle64(richards_ctx* c, int l, bool d_ready = false) {
   const int model = c->soil.model;
   const Phys<double> P = phys<double>(c);
-  if (l >= c->tail_start) {
+  if (l >= c->team_start64) {
     Prof pr(c, "tail64", l, c->L[l].ncell);
-    rich::tail64(c->dL64, c->dX64, l, c->nlev, P, model, c->opts.nu1, c->opts.nu2, c->opts.coarse_max_sweeps,
-                 c->opts.coarse_rtol, c->opts.cycle_gamma, c->opts.gamma_levels, c->scratch + 16, c->opts.ordering,
+    rich::tail64(c->dL64, c->dX64, l, c->nlev, tail_shape<double>(c, l), P, model, c->opts.nu1, c->opts.nu2,
+                 c->opts.coarse_max_sweeps, c->opts.coarse_rtol, c->opts.cycle_gamma, c->opts.gamma_levels, c->scratch + 16, c->opts.ordering,
                  c->s);
     return;
   }
@@ -660,10 +683,10 @@ void vcycle32(richards_ctx* c, int l, bool d_ready = false, bool fuse = false) {
     c->graph_err = std::string("cooperative launch: ") + cudaGetErrorString(e);
     c->coop_start = MAXLEV;
   }
-  if (l >= c->tail_start) {
+  if (l >= c->team_start32) {
     Prof pr(c, "tail32", l, c->L[l].ncell);
-    rich::tail32(c->dL32, c->dX32, l, c->nlev, P, model, c->opts.nu1, c->opts.nu2, c->opts.coarse_max_sweeps,
-                 (float)c->opts.coarse_rtol, c->opts.cycle_gamma, c->opts.gamma_levels, c->scratch + 16,
+    rich::tail32(c->dL32, c->dX32, l, c->nlev, tail_shape<float>(c, l), P, model, c->opts.nu1, c->opts.nu2,
+                 c->opts.coarse_max_sweeps, (float)c->opts.coarse_rtol, c->opts.cycle_gamma, c->opts.gamma_levels, c->scratch + 16,
                  c->opts.ordering, c->s);
     return;
   }
@@ -1389,9 +1412,12 @@ void batch_tail(richards_batcher* b, std::vector<BatchCtx>& B, const std::vector
   const richards_opts& o = B[who[0]].c->opts;
   for (size_t a = 0; a < who.size(); a += rich::BATCH_MAX) {
     rich::BList list{};
-    for (size_t q = a; q < who.size() && q < a + rich::BATCH_MAX; ++q)
+    int blocks = 1;                   // (one size a launch: the biggest level's)
+    for (size_t q = a; q < who.size() && q < a + rich::BATCH_MAX; ++q) {
       list.job[list.n++] = B[who[q]].slot * MAXLEV + l;
-    rich::batch_tail32(b->dtable, list, o.nu1, o.nu2, o.coarse_max_sweeps, (float)o.coarse_rtol, o.cycle_gamma,
+      blocks = std::max(blocks, tail_shape<float>(B[who[q]].c, l).blocks);
+    }
+    rich::batch_tail32(b->dtable, list, blocks, o.nu1, o.nu2, o.coarse_max_sweeps, (float)o.coarse_rtol, o.cycle_gamma,
                        o.gamma_levels, b->s);
   }
 }
@@ -1408,7 +1434,7 @@ void batch_smooth(richards_batcher* b, std::vector<BatchCtx>& B, const std::vect
 // solve, where a context whose stop test left the defect in place skips it)
 void batch_vcycle(richards_batcher* b, std::vector<BatchCtx>& B, const std::vector<int>& who, int l, bool top) {
   std::vector<int> tail, grid;
-  for (int k : who) (l >= B[k].c->tail_start ? tail : grid).push_back(k);
+  for (int k : who) (l >= B[k].c->team_start_batch ? tail : grid).push_back(k);
   if (!tail.empty()) batch_tail(b, B, tail, l);
   if (grid.empty()) return;
   const richards_opts& o = B[grid[0]].c->opts;
@@ -1490,6 +1516,9 @@ void batch_table_slot(richards_batcher* b, std::vector<BatchCtx>& B, int k) {
     J.dXs = c->dX32;
     J.level = l;
     J.nlev = c->nlev;
+    const rich::TeamShape ts = tail_shape<float>(c, l);
+    J.tail_start = ts.tail_start;
+    J.handoff = ts.handoff;
     J.model = c->soil.model;
     J.norm = b->dnorm + B[k].slot;
     J.stats = c->scratch + 16;
@@ -1800,6 +1829,9 @@ richards_status richards_create(const richards_grid* grid, const richards_opts* 
   for (int l = 0; l < c->nlev; ++l)
     if ((long long)c->L[l].n[0] * c->L[l].n[1] * c->L[l].n[2] <= o.tail_cells) { c->tail_start = l; break; }
   const bool mixed = o.precision >= 1;
+  c->team_start64 = team_start<double>(c);
+  c->team_start32 = team_start<float>(c);
+  c->team_start_batch = team_start<float>(c, true);
   c->coop_start = MAXLEV;
   if (o.precision >= 1 && COOP_CELLS > 0)
     for (int l = 1; l < c->tail_start; ++l)

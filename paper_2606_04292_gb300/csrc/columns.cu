@@ -52,6 +52,14 @@ struct ColArgs {
       model;
 };
 
+// what the inner solve of a column reads of its physics and options (in
+// shared memory)
+struct ColShared {
+  Phys<float> P;
+  int nu1, nu2, cmax, gamma, gamma_levels, inner_cycles;
+  float crtol, inner_rtol;
+};
+
 // 1D hierarchy of one column in shared memory; transfer weights computed on
 // the fly (columns have arbitrary lengths, nf -> nc = ceil(nf/2)): the coarse
 // coordinate of fine cell i is num/den = ((2i+1) nc - nf)/(2 nf), so with the
@@ -118,9 +126,34 @@ struct ColumnLevels {
   }
 };
 
+// One inner solve of a column: cycles until the defect is at most inner_rtol
+// rin0 or the limit is reached; returns the cycles done and adds their updates
+// to *updates.  A function of its own, with the physics in shared memory: the
+// outer layer's FP64 and float-float constants (some 90 registers) are then
+// not live across the cycle, which otherwise spilled (4096 columns x 4 steps:
+// 71.8 ms inlined).
+template <int MODEL>
+__device__ __noinline__ int column_inner(const Level<float>* Ls, float slo, float shi, int nl, const ColShared* S,
+                                         float rin0, unsigned long long* sm, unsigned long long* updates) {
+  BlockTeam tm{sm};
+  const ColumnLevels lv{Ls, slo, shi};
+  unsigned long long up = 0;
+  int k = 0;
+  for (;;) {
+    team_cycle<float, FORM_DELTA, MODEL>(lv, 0, nl, S->P, S->nu1, S->nu2, S->cmax, S->crtol, S->gamma, S->gamma_levels,
+                                         up, 1, nl, tm);
+    ++k;
+    if (k >= S->inner_cycles) break;
+    if (S->inner_rtol > 0.0f && team_defect<float, FORM_DELTA, MODEL>(Ls[0], S->P, false, tm) <= S->inner_rtol * rin0)
+      break;
+  }
+  *updates += up;
+  return k;
+}
+
 template <int MODEL>
 __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>* Ls, int* s_nl, double* kb64,
-                             unsigned long long* sm) {
+                             unsigned long long* sm, ColShared* S) {
   const ColDesc D = A.cols[c];
   const int n = D.n;
   const long long off = D.off;
@@ -165,11 +198,18 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
   P64.p1 = D.p1; P64.p2 = D.p2; P64.p3 = D.p3; P64.p4 = D.p4;
   P64.h1 = A.h1; P64.h2 = A.h2; P64.h3 = A.h3; P64.h4 = A.h4;
   P64.newton_k = A.newton_k; P64.sink = A.sink; P64.lag = A.lag;
-  Phys<float> P32{};
-  P32.xi = (float)A.xi; P32.kappa = (float)A.kappa; P32.ts = (float)D.ts; P32.tr = (float)D.tr;
-  P32.p1 = (float)D.p1; P32.p2 = (float)D.p2; P32.p3 = (float)D.p3; P32.p4 = (float)D.p4;
-  P32.h1 = (float)A.h1; P32.h2 = (float)A.h2; P32.h3 = (float)A.h3; P32.h4 = (float)A.h4;
-  P32.newton_k = A.newton_k; P32.sink = A.sink; P32.lag = A.lag;
+  if (threadIdx.x == 0) {              // (read after the barriers of the step's preparation)
+    Phys<float> P32{};
+    P32.xi = (float)A.xi; P32.kappa = (float)A.kappa; P32.ts = (float)D.ts; P32.tr = (float)D.tr;
+    P32.p1 = (float)D.p1; P32.p2 = (float)D.p2; P32.p3 = (float)D.p3; P32.p4 = (float)D.p4;
+    P32.h1 = (float)A.h1; P32.h2 = (float)A.h2; P32.h3 = (float)A.h3; P32.h4 = (float)A.h4;
+    P32.newton_k = A.newton_k; P32.sink = A.sink; P32.lag = A.lag;
+    S->P = P32;
+    S->nu1 = A.nu1; S->nu2 = A.nu2; S->cmax = A.cmax; S->gamma = A.gamma; S->gamma_levels = A.gamma_levels;
+    S->inner_cycles = A.inner_cycles;
+    S->crtol = (float)A.crtol;
+    S->inner_rtol = (float)A.inner_rtol;
+  }
   double* psin = A.psin + off;
   double* psinm1 = A.psinm1 + off;
   double* thn = A.thn + off;
@@ -193,7 +233,7 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
     const int scheme = (A.scheme == 2 && have_prev) ? 2 : 1;
     const double a = scheme == 1 ? 1.0 / A.dt : 1.5 / A.dt;
     P64.a = a;
-    P32.a = (float)a;
+    if (threadIdx.x == 0) S->P.a = (float)a;
     const DDPhys Q = make_ddphys_dev(P64);
     const dd Ks = dd_split(D.Ks);
     const dd hist_scale = dd_split(scheme == 1 ? 1.0 / A.dt : 1.0 / (2.0 * A.dt));
@@ -370,16 +410,7 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
           const_cast<float*>(Ls[l + 1].psi0)[J] = lv.restrict(l, Ls[l].psi0, J, 0, 0);
         __syncthreads();
       }
-      const float rin0 = (float)nrm;
-      for (int k = 0; k < A.inner_cycles; ++k) {
-        block_cycle<float, FORM_DELTA, MODEL>(lv, 0, nl, P32, A.nu1, A.nu2, A.cmax, (float)A.crtol, A.gamma,
-                                              A.gamma_levels, sm, updates);
-        ++cyc_total;
-        if (A.inner_rtol > 0.0 && k + 1 < A.inner_cycles) {
-          const float rin = block_defect_norm<float, FORM_DELTA, MODEL>(Ls[0], P32, sm);
-          if (rin <= (float)A.inner_rtol * rin0) break;
-        }
-      }
+      cyc_total += column_inner<MODEL>(Ls, lv.slo, lv.shi, nl, S, (float)nrm, sm, &updates);
       for (int i = threadIdx.x; i < n; i += blockDim.x) G.u[i] += (double)Ls[0].u[i];
       __syncthreads();
       ++outer;
@@ -413,6 +444,7 @@ __global__ void __launch_bounds__(COL_THREADS_MAX, 1) k_columns(ColArgs A) {
   __shared__ Level<float> Ls[COL_MAXLEV];
   __shared__ unsigned long long sm[33];
   __shared__ double kb64[2];
+  __shared__ ColShared S;
   __shared__ int s_col, s_nl;
   for (;;) {
     if (threadIdx.x == 0) {
@@ -423,7 +455,7 @@ __global__ void __launch_bounds__(COL_THREADS_MAX, 1) k_columns(ColArgs A) {
     const int c = s_col;
     __syncthreads();
     if (c < 0) break;
-    column_solve<MODEL>(A, c, smem, Ls, &s_nl, kb64, sm);
+    column_solve<MODEL>(A, c, smem, Ls, &s_nl, kb64, sm, &S);
   }
 }
 

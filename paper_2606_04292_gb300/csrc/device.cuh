@@ -922,6 +922,32 @@ __device__ __forceinline__ T restrict_at(const Level<T>& F, const Xfer<T>& X, co
   return s;
 }
 
+// two natural-layout arrays through one reading of the tables (the sums of
+// restrict_at)
+template <typename T>
+__device__ __forceinline__ void restrict2_at(const Level<T>& F, const Xfer<T>& X, const T* __restrict__ fa,
+                                             const T* __restrict__ fb, int J0, int J1, int J2, T& a, T& b) {
+  T sa = T(0), sb = T(0);
+  const int c0 = X.rc[0][J0], c1 = X.rc[1][J1], c2 = X.rc[2][J2];
+  for (int a2 = 0; a2 < c2; ++a2) {
+    const int f2 = X.ri[2][RMAX * J2 + a2];
+    const T w2 = X.rw[2][RMAX * J2 + a2];
+    for (int a1 = 0; a1 < c1; ++a1) {
+      const int f1 = X.ri[1][RMAX * J1 + a1];
+      const T w1 = X.rw[1][RMAX * J1 + a1];
+      const long long row = (long long)F.n0 * (f1 + (long long)F.n1 * f2);
+      for (int a0 = 0; a0 < c0; ++a0) {
+        const T w0 = X.rw[0][RMAX * J0 + a0];
+        const long long idx = row + X.ri[0][RMAX * J0 + a0];
+        sa += w0 * w1 * w2 * fa[idx];
+        sb += w0 * w1 * w2 * fb[idx];
+      }
+    }
+  }
+  a = sa;
+  b = sb;
+}
+
 // sum_J P(i, J) (u_c - ubar_c)(J)
 template <typename T>
 __device__ __forceinline__ T prolong_at(const Level<T>& C, const Xfer<T>& X, int i0, int i1, int i2) {

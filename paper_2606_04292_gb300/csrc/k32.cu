@@ -16,10 +16,11 @@ void restrict32(const Level<float>& F, const Level<float>& C, const Xfer<float>&
 void prolong32(const Level<float>& F, const Level<float>& C, const Xfer<float>& X, cudaStream_t s) {
   D::prolong(F, C, X, s);
 }
-void tail32(const Level<float>* dLs, const Xfer<float>* dXs, int l0, int nl, const Phys<float>& P, int model,
+void tail32(const Level<float>* dLs, const Xfer<float>* dXs, int l0, int nl, const TeamShape& ts,
+            const Phys<float>& P, int model,
             int nu1, int nu2, int cmax, float crtol, int gamma, int gamma_levels, unsigned long long* stats,
             int ordering, cudaStream_t s) {
-  D::tail(dLs, dXs, l0, nl, P, model, nu1, nu2, cmax, crtol, gamma, gamma_levels, stats, ordering, s);
+  D::tail(dLs, dXs, l0, nl, ts, P, model, nu1, nu2, cmax, crtol, gamma, gamma_levels, stats, ordering, s);
 }
 int coop_max_blocks32(int model) { return D::coop_max_blocks(model); }
 cudaError_t coop32(const Level<float>* dLs, const Xfer<float>* dXs, int l0, int nl, int tail_start,

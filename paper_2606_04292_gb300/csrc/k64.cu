@@ -20,10 +20,11 @@ void restrict64(const Level<double>& F, const Level<double>& C, const Xfer<doubl
 void prolong64(const Level<double>& F, const Level<double>& C, const Xfer<double>& X, cudaStream_t s) {
   D::prolong(F, C, X, s);
 }
-void tail64(const Level<double>* dLs, const Xfer<double>* dXs, int l0, int nl, const Phys<double>& P, int model,
+void tail64(const Level<double>* dLs, const Xfer<double>* dXs, int l0, int nl, const TeamShape& ts,
+            const Phys<double>& P, int model,
             int nu1, int nu2, int cmax, double crtol, int gamma, int gamma_levels, unsigned long long* stats,
             int ordering, cudaStream_t s) {
-  D::tail(dLs, dXs, l0, nl, P, model, nu1, nu2, cmax, crtol, gamma, gamma_levels, stats, ordering, s);
+  D::tail(dLs, dXs, l0, nl, ts, P, model, nu1, nu2, cmax, crtol, gamma, gamma_levels, stats, ordering, s);
 }
 void sweep_lex64(const Level<double>& L, const Phys<double>& P, int model, cudaStream_t s) { D::sweep_lex(L, P, model, s); }
 

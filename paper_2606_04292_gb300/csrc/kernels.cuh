@@ -488,33 +488,108 @@ __host__ __device__ inline bool nested_levels(int fn0, int fn1, int fn2, int cn0
 }
 
 // ---------------------------------------------------------------------------
-// The coarse tail: the whole V-cycle from level l0 down to the coarsest level
-// in one thread block (levels small enough that launch latency would dominate
-// a kernel per stage).  Same arithmetic as the grid kernels, phase by phase,
-// separated by block barriers.
-// ---------------------------------------------------------------------------
+// The coarse tail: the whole cycle from level l0 down in one launch (levels
+// small enough that launch latency would dominate a kernel per stage).  Same
+// arithmetic as the grid kernels, phase by phase, separated by barriers.
+//
 // The cycle's loops run over a "team" of threads: one thread block (the
-// coarse tail, the batched columns, the single-block step) or every thread of
-// a cooperative grid (the coarse levels of a big grid: no launch per stage).
-// rank/size index the team's threads, sync() is its barrier, max() its
-// max-reduction (every thread gets the result).
+// batched columns), the blocks of one thread-block cluster (the coarse tail,
+// the small-grid step), or every block of a cooperative grid.  rank/size index
+// the team's threads, sync() is its barrier, max() its max-reduction (every
+// thread gets the result).  A team of several blocks can hand the smallest
+// levels to its first block alone (solo: block barriers), while the others
+// wait at the team's next barrier.
+//
+// Why a cluster: a phase of a 64^2 level is 2048 point updates, which one SM
+// issues in ~5.5 us (FP32) or, bound by its FP64 pipe, ~40 us (FP64); spread
+// over 16 SMs it takes the latency of one update, and the hardware barrier of
+// a cluster costs a fraction of a launch or of a grid-wide barrier.
+// ---------------------------------------------------------------------------
 struct BlockTeam {
+  static constexpr bool splits = false;
+  unsigned long long* sm;              // 33 words
   __device__ unsigned rank() const { return threadIdx.x; }
   __device__ unsigned size() const { return blockDim.x; }
   __device__ void sync() const { __syncthreads(); }
-  __device__ unsigned long long max(unsigned long long v, unsigned long long* sm) const { return block_max(v, sm); }
+  __device__ unsigned long long max(unsigned long long v) const { return block_max(v, sm); }
+};
+
+// Shared memory of a cluster team: block_max's words and two rotating rows of
+// one maximum per block.
+constexpr int CLUSTER_MAX = 16;
+struct ClusterShared {
+  unsigned long long sm[33];
+  unsigned long long part[2][CLUSTER_MAX];
+};
+
+// The blocks of one cluster (1 to CLUSTER_MAX).  Warps are dealt round robin
+// over the blocks, so that a level with few cells uses every SM of the
+// cluster.  (barrier.cluster releases and acquires at cluster scope: global
+// memory written before it by any block is visible after it to all.)
+struct ClusterTeam {
+  static constexpr bool splits = true;
+  ClusterShared* sh;
+  unsigned nct, ct;
+  bool solo;
+  int parity;
+  __device__ explicit ClusterTeam(ClusterShared* s) : sh(s), parity(0) {
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nct));
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(ct));
+    solo = nct == 1;
+  }
+  __device__ bool lead() const { return ct == 0; }
+  __device__ unsigned rank() const {
+    return solo ? threadIdx.x : (((threadIdx.x >> 5) * nct + ct) << 5) + (threadIdx.x & 31);
+  }
+  __device__ unsigned size() const { return solo ? blockDim.x : blockDim.x * nct; }
+  __device__ void cluster_sync() const {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  __device__ void sync() const {
+    if (solo) __syncthreads();
+    else cluster_sync();
+  }
+  // (every block writes its maximum into every block's row; the row is next
+  // written two reductions, and so at least one cluster barrier, later)
+  __device__ unsigned long long max(unsigned long long v) {
+    v = block_max(v, sh->sm);
+    if (solo) return v;
+    if (threadIdx.x < nct) {
+      const unsigned a = (unsigned)__cvta_generic_to_shared(&sh->part[parity][ct]);
+      unsigned r;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(threadIdx.x));
+      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(r), "l"(v) : "memory");
+    }
+    cluster_sync();
+    unsigned long long m = 0;
+    for (unsigned k = 0; k < nct; ++k) {
+      const unsigned long long w = sh->part[parity][k];
+      m = w > m ? w : m;
+    }
+    parity ^= 1;
+    return m;
+  }
 };
 
 // (three global slots rotate: the slot zeroed at one reduction was last read
 // two reductions earlier, with a grid barrier in between)
 struct GridTeam {
+  static constexpr bool splits = true;
   unsigned long long* slots;
+  unsigned long long* sm;
   int round;
-  __device__ unsigned rank() const { return blockIdx.x * blockDim.x + threadIdx.x; }
-  __device__ unsigned size() const { return gridDim.x * blockDim.x; }
-  __device__ void sync() const { cooperative_groups::this_grid().sync(); }
-  __device__ unsigned long long max(unsigned long long v, unsigned long long* sm) {
+  bool solo;
+  __device__ bool lead() const { return blockIdx.x == 0; }
+  __device__ unsigned rank() const { return solo ? threadIdx.x : blockIdx.x * blockDim.x + threadIdx.x; }
+  __device__ unsigned size() const { return solo ? blockDim.x : gridDim.x * blockDim.x; }
+  __device__ void sync() const {
+    if (solo) __syncthreads();
+    else cooperative_groups::this_grid().sync();
+  }
+  __device__ unsigned long long max(unsigned long long v) {
     v = block_max(v, sm);
+    if (solo) return v;
     unsigned long long* s = slots + round % 3;
     if (threadIdx.x == 0) atomicMax(s, v);
     if (rank() == 0) slots[(round + 1) % 3] = 0ull;
@@ -526,48 +601,51 @@ struct GridTeam {
 };
 
 // one NGS sweep of a level by a team: red then black half-sweeps (ordering
-// 1), or the lexicographic order hyperplane by hyperplane (0)
-template <typename T, int FORM, int MODEL, typename TM = BlockTeam>
-__device__ __forceinline__ void block_sweep(const Level<T>& L, const Phys<T>& P, int ordering = 1, TM tm = TM{}) {
-  if (ordering == 0) {
-    const int nplanes = L.n0 + L.n1 + L.n2 - 2;
-    const int nrows = L.n1 * L.n2;
-    for (int s = 0; s < nplanes; ++s) {
-      for (int t = tm.rank(); t < nrows; t += tm.size()) {
-        const int i2 = (int)quick_div((unsigned)t, (unsigned)L.n1, L.rn1), i1 = t - i2 * L.n1;
-        const int i0 = s - i1 - i2;
-        if (i0 >= 0 && i0 < L.n0)
-          point_update<T, FORM, MODEL>(L, P, (unsigned)(i0 + L.n0 * t), i0, i1, i2);
-      }
-      tm.sync();
-    }
-    return;
-  }
-  const unsigned nh = (unsigned)((L.n0 + 1) >> 1) * (unsigned)L.n1 * (unsigned)L.n2;
-  for (int color = 0; color < 2; ++color) {
-    for (unsigned t = tm.rank(); t < nh; t += tm.size()) {
+// 1), or the lexicographic order hyperplane by hyperplane (0).  One copy of
+// the point update serves both.
+template <typename T, int FORM, int MODEL, typename TM>
+__device__ __forceinline__ void team_sweep(const Level<T>& L, const Phys<T>& P, int ordering, TM& tm) {
+  const unsigned rows = (unsigned)L.n1 * (unsigned)L.n2;
+  const unsigned items = ordering ? (unsigned)((L.n0 + 1) >> 1) * rows : rows;
+  const int phases = ordering ? 2 : L.n0 + L.n1 + L.n2 - 2;
+  for (int ph = 0; ph < phases; ++ph) {
+    for (unsigned t = tm.rank(); t < items; t += tm.size()) {
       int i0, i1, i2;
       unsigned i;
-      if (color_cell(L, t, color, i0, i1, i2, i)) point_update<T, FORM, MODEL>(L, P, i, i0, i1, i2);
+      bool on;
+      if (ordering) {
+        on = color_cell(L, t, ph, i0, i1, i2, i);
+      } else {
+        i2 = (int)quick_div(t, (unsigned)L.n1, L.rn1);
+        i1 = (int)t - i2 * L.n1;
+        i0 = ph - i1 - i2;
+        on = i0 >= 0 && i0 < L.n0;
+        i = (unsigned)i0 + (unsigned)L.n0 * t;
+      }
+      if (on) point_update<T, FORM, MODEL>(L, P, i, i0, i1, i2);
     }
     tm.sync();
   }
 }
 
-template <typename T, int FORM, int MODEL, typename TM = BlockTeam>
-__device__ __forceinline__ T block_defect_norm(const Level<T>& L, const Phys<T>& P, unsigned long long* sm,
-                                               TM* tmp = nullptr) {
-  TM local{};
-  TM& tm = tmp ? *tmp : local;
+// the defect d = g - N(u) of a level by a team: stored (store), or its
+// max-norm (returned to every thread)
+template <typename T, int FORM, int MODEL, typename TM>
+__device__ __forceinline__ T team_defect(const Level<T>& L, const Phys<T>& P, bool store, TM& tm) {
   unsigned long long mx = 0;
-  for (long long i = tm.rank(); i < L.ncell; i += tm.size()) {
+  for (unsigned i = tm.rank(); i < (unsigned)L.ncell; i += tm.size()) {
     int i0, i1, i2;
-    cell_coords(L, (unsigned)i, i0, i1, i2);
+    cell_coords(L, i, i0, i1, i2);
     const T di = L.g[pix(L, i, i0, i1, i2)] - apply_N<T, FORM, MODEL>(L, P, L.u, i, i0, i1, i2);
+    if (store) L.d[i] = di;
     const unsigned long long b = nbits(di);
     mx = b > mx ? b : mx;
   }
-  return from_bits<T>(tm.max(mx, sm));
+  if (store) {
+    tm.sync();
+    return T(0);
+  }
+  return from_bits<T>(tm.max(mx));
 }
 
 // Levels l0..nl-1 of one multigrid cycle by one team, with the recursion of
@@ -576,155 +654,171 @@ __device__ __forceinline__ T block_defect_norm(const Level<T>& L, const Phys<T>&
 // W-cycle); the coarsest level sweeps until its defect drops by crtol or
 // cmax sweeps are done; prolongation and post-smoothing on the way up.  LV
 // gives the level views (L(l)) and the transfers from level l:
-// restrict(l, fine array, coarse coords) and prolong(l, fine coords).
-// (handoff < nl, grid teams only: from level handoff on, block 0 alone runs
-// the rest of the cycle with block barriers, as the single-block tail does,
-// while the other blocks wait at the next grid barrier; tail_lv gives that
-// part's levels and transfers)
-template <typename T, int FORM, int MODEL>
-struct NoTail {};
-
-template <typename T, int FORM, int MODEL, typename LV, typename TM = BlockTeam, typename TLV = NoTail<T, FORM, MODEL>>
-__device__ __forceinline__ void block_cycle(const LV& lv, int l0, int nl, const Phys<T>& P, int nu1, int nu2, int cmax, T crtol,
-                            int gamma, int gamma_levels, unsigned long long* sm, unsigned long long& updates,
-                            int ordering = 1, TM* tmp = nullptr, int handoff = 1 << 30,
-                            const TLV* tail_lv = nullptr) {
-  TM local{};
-  TM& tm = tmp ? *tmp : local;
-  int visits[24];
-  int l = l0;
-  bool down = true;
+// restrict2(l, fine arrays, coarse coords) and prolong(l, fine coords).
+// handoff (teams of several blocks): levels from handoff on run solo.
+// One loop, with one copy of the sweep, the defect and the FAS right side:
+// the busy warps of a small level fetch each instruction for themselves, and
+// a copy per use was a fifth of their stall cycles.
+template <typename T, int FORM, int MODEL, typename LV, typename TM>
+__device__ __forceinline__ void team_cycle(const LV& lv, int l0, int nl, const Phys<T>& P, int nu1, int nu2, int cmax,
+                                           T crtol, int gamma, int gamma_levels, unsigned long long& updates,
+                                           int ordering, int handoff, TM& tm) {
+  enum { DOWN, COARSEST, POST };
+  unsigned long long visits = 0;         // coarse visits done from each level, two bits a level (gamma <= 3)
+  int l = l0, solo_at = -1;
+  bool arrive = true;                    // at level l from above
+  int stage = DOWN, sweeps = 0, done = 0;
+  T d0 = T(0);
   for (;;) {
-    if (down) {
-      if constexpr (!std::is_same<TLV, NoTail<T, FORM, MODEL>>::value) {
-        if (l == handoff) {
-          if (blockIdx.x == 0)
-            block_cycle<T, FORM, MODEL, TLV>(*tail_lv, l, nl, P, nu1, nu2, cmax, crtol, gamma, gamma_levels, sm,
-                                             updates, ordering);
-          tm.sync();
-          down = false;
-          continue;
+    bool finished = false;
+    if (arrive) {
+      arrive = false;
+      if constexpr (TM::splits) {
+        if (!tm.solo && l >= handoff) {
+          if (tm.lead()) {
+            tm.solo = true;
+            solo_at = l;
+          } else {
+            tm.sync();                   // (the first block's, when it has finished level l)
+            finished = true;
+          }
         }
       }
-      if (l == nl - 1) {
-        const Level<T>& C = lv.L(l);
-        const T d0 = block_defect_norm<T, FORM, MODEL, TM>(C, P, sm, &tm);
-        for (int s = 0; s < cmax; ++s) {
-          block_sweep<T, FORM, MODEL, TM>(C, P, ordering, tm);
-          updates += C.ncell;
-          const T dn = block_defect_norm<T, FORM, MODEL, TM>(C, P, sm, &tm);
-          if (!(dn > crtol * d0)) break;
+      stage = l == nl - 1 ? COARSEST : DOWN;
+      sweeps = stage == COARSEST ? (cmax > 1 ? 0 : 1) : nu1;
+      done = 0;
+    }
+    if (!finished) {
+      const Level<T>& F = lv.L(l);
+      for (int s = 0; s < sweeps; ++s) team_sweep<T, FORM, MODEL, TM>(F, P, ordering, tm);
+      updates += (unsigned long long)sweeps * F.ncell;
+      finished = true;
+      if (stage == COARSEST) {
+        done += sweeps;
+        if (done < cmax) {               // (the last sweep's defect would change nothing)
+          const T dn = team_defect<T, FORM, MODEL, TM>(F, P, false, tm);
+          if (done == 0) d0 = dn;
+          finished = done > 0 && !(dn > crtol * d0);
+          sweeps = 1;
         }
-        down = false;
+        if (!finished) continue;
+      } else if (stage == DOWN) {
+        team_defect<T, FORM, MODEL, TM>(F, P, true, tm);
+        const Level<T>& C = lv.L(l + 1);
+        for (unsigned J = tm.rank(); J < (unsigned)C.ncell; J += tm.size()) {
+          int J0, J1, J2;
+          cell_coords(C, J, J0, J1, J2);
+          lv.restrict2(l, F.u, F.d, J0, J1, J2, C.ubar[J], C.d[J]);
+        }
+        tm.sync();
+        for (unsigned J = tm.rank(); J < (unsigned)C.ncell; J += tm.size()) {
+          int J0, J1, J2;
+          cell_coords(C, J, J0, J1, J2);
+          C.g[J] = apply_N<T, FORM, MODEL>(C, P, C.ubar, J, J0, J1, J2) + C.d[J];
+          C.u[J] = C.ubar[J];
+        }
+        tm.sync();
+        visits &= ~(3ull << (2 * l));
+        ++l;
+        arrive = true;
         continue;
       }
-      const Level<T>& F = lv.L(l);
-      for (int s = 0; s < nu1; ++s) block_sweep<T, FORM, MODEL, TM>(F, P, ordering, tm);
-      updates += (unsigned long long)nu1 * F.ncell;
-      for (long long i = tm.rank(); i < F.ncell; i += tm.size()) {
-        int i0, i1, i2;
-        cell_coords(F, (unsigned)i, i0, i1, i2);
-        F.d[i] = F.g[pix(F, i, i0, i1, i2)] - apply_N<T, FORM, MODEL>(F, P, F.u, i, i0, i1, i2);
-      }
-      tm.sync();
-      const Level<T>& C = lv.L(l + 1);
-      for (long long J = tm.rank(); J < C.ncell; J += tm.size()) {
-        int J0, J1, J2;
-        cell_coords(C, (unsigned)J, J0, J1, J2);
-        lv.restrict2(l, F.u, F.d, J0, J1, J2, C.ubar[J], C.d[J]);
-      }
-      tm.sync();
-      for (long long J = tm.rank(); J < C.ncell; J += tm.size()) {
-        int J0, J1, J2;
-        cell_coords(C, (unsigned)J, J0, J1, J2);
-        C.g[J] = apply_N<T, FORM, MODEL>(C, P, C.ubar, J, J0, J1, J2) + C.d[J];
-        C.u[J] = C.ubar[J];
-      }
-      tm.sync();
-      visits[l] = 0;
-      ++l;
-      continue;
     }
     // level l is finished: back to its parent
+    if constexpr (TM::splits) {
+      if (solo_at == l) {
+        solo_at = -1;
+        tm.solo = false;
+        tm.sync();
+      }
+    }
     if (l == l0) break;
     const int pl = l - 1;
     const int g = (gamma_levels <= 0 || pl < gamma_levels) ? gamma : 1;
-    if (++visits[pl] < g) {           // visit the coarser level again (same right side)
-      l = pl + 1;
-      down = true;
+    visits += 1ull << (2 * pl);
+    if ((int)((visits >> (2 * pl)) & 3) < g) {           // visit the coarser level again (same right side)
+      arrive = true;
       continue;
     }
     const Level<T>& F = lv.L(pl);
-    for (long long i = tm.rank(); i < F.ncell; i += tm.size()) {
+    for (unsigned i = tm.rank(); i < (unsigned)F.ncell; i += tm.size()) {
       int i0, i1, i2;
-      cell_coords(F, (unsigned)i, i0, i1, i2);
+      cell_coords(F, i, i0, i1, i2);
       F.u[i] += lv.prolong(pl, i0, i1, i2);
     }
     tm.sync();
-    for (int s = 0; s < nu2; ++s) block_sweep<T, FORM, MODEL, TM>(F, P, ordering, tm);
-    updates += (unsigned long long)nu2 * F.ncell;
     l = pl;
+    stage = POST;
+    sweeps = nu2;
   }
 }
 
+// The levels of a cycle as the grid kernels treat them: above the coarse
+// tail's first level the transfers take the nested formulas where the levels
+// nest and the tables otherwise, from it on the tables, so that a launch of
+// several levels gives the values of the launches it replaces.
 template <typename T>
-struct DeviceLevels {
-  const Level<T>* Ls;
+struct GridLevels {
+  const Level<T>* Ls;                  // views and tables of levels base, base + 1, ...
   const Xfer<T>* Xs;
-  __device__ const Level<T>& L(int l) const { return Ls[l]; }
-  __device__ T restrict(int l, const T* fine, int J0, int J1, int J2) const {
-    return restrict_at(Ls[l], Xs[l], fine, J0, J1, J2);
-  }
-  __device__ void restrict2(int l, const T* fa, const T* fb, int J0, int J1, int J2, T& a, T& b) const {
-    a = restrict(l, fa, J0, J1, J2);
-    b = restrict(l, fb, J0, J1, J2);
-  }
-  __device__ T prolong(int l, int i0, int i1, int i2) const { return prolong_at(Ls[l + 1], Xs[l], i0, i1, i2); }
-};
-
-template <typename T, int FORM, int MODEL>
-__global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail(const Level<T>* __restrict__ Ls, const Xfer<T>* __restrict__ Xs,
-                                                       int l0, int nl, Phys<T> P, int nu1, int nu2, int cmax,
-                                                       T crtol, int gamma, int gamma_levels, unsigned long long* stats,
-                                                       int ordering) {
-  __shared__ unsigned long long sm[33];
-  unsigned long long updates = 0;
-  block_cycle<T, FORM, MODEL>(DeviceLevels<T>{Ls, Xs}, l0, nl, P, nu1, nu2, cmax, crtol, gamma, gamma_levels, sm,
-                              updates, ordering);
-  if (threadIdx.x == 0 && stats) atomicAdd(stats, updates);
-}
-
-// The coarse levels of a big grid as one cooperative launch: block_cycle run
-// by every thread of the grid, a grid barrier between phases instead of a
-// launch per stage.  Above the single-block tail's first level the transfers
-// are the grid kernels' (nested formulas where the levels nest, tables
-// otherwise), from it on the tail's (tables): the values equal those of the
-// launches it replaces.
-template <typename T>
-struct CoopLevels {
-  const Level<T>* Ls;
-  const Xfer<T>* Xs;
-  int tail_start;
-  __device__ const Level<T>& L(int l) const { return Ls[l]; }
+  int base, tail_start;
+  __device__ const Level<T>& L(int l) const { return Ls[l - base]; }
   __device__ bool nested(int l) const {
-    const Level<T>& F = Ls[l];
-    const Level<T>& C = Ls[l + 1];
+    const Level<T>& F = L(l);
+    const Level<T>& C = L(l + 1);
     return l < tail_start && nested_levels(F.n0, F.n1, F.n2, C.n0, C.n1, C.n2);
   }
-  __device__ T restrict(int l, const T* fine, int J0, int J1, int J2) const {
-    return nested(l) ? restrict_nested_at(Ls[l], Ls[l + 1], fine, J0, J1, J2)
-                     : restrict_at(Ls[l], Xs[l], fine, J0, J1, J2);
-  }
   __device__ void restrict2(int l, const T* fa, const T* fb, int J0, int J1, int J2, T& a, T& b) const {
-    a = restrict(l, fa, J0, J1, J2);
-    b = restrict(l, fb, J0, J1, J2);
+    if (nested(l)) {
+      a = restrict_nested_at(L(l), L(l + 1), fa, J0, J1, J2);
+      b = restrict_nested_at(L(l), L(l + 1), fb, J0, J1, J2);
+    } else {
+      restrict2_at(L(l), Xs[l - base], fa, fb, J0, J1, J2, a, b);
+    }
   }
   __device__ T prolong(int l, int i0, int i1, int i2) const {
-    return nested(l) ? prolong_nested_at(Ls[l], Ls[l + 1], Xs[l], i0, i1, i2) : prolong_at(Ls[l + 1], Xs[l], i0, i1, i2);
+    return nested(l) ? prolong_nested_at(L(l), L(l + 1), Xs[l - base], i0, i1, i2)
+                     : prolong_at(L(l + 1), Xs[l - base], i0, i1, i2);
   }
 };
 
-// slots: three global words for the grid reductions; stats: the update count
+// copies the descriptors of levels l0 .. nl - 1 to shared memory (the blocks
+// read them in every phase; ends without a barrier)
+template <typename T>
+__device__ __forceinline__ void stage_levels(const Level<T>* Ls, const Xfer<T>* Xs, int l0, int nl, Level<T>* sL,
+                                             Xfer<T>* sX) {
+  static_assert(sizeof(Level<T>) % 4 == 0 && sizeof(Xfer<T>) % 4 == 0, "copied as words");
+  const unsigned* a = reinterpret_cast<const unsigned*>(Ls + l0);
+  const unsigned* b = reinterpret_cast<const unsigned*>(Xs + l0);
+  const int na = (int)(sizeof(Level<T>) / 4) * (nl - l0), nb = (int)(sizeof(Xfer<T>) / 4) * (nl - l0);
+  for (int k = threadIdx.x; k < na; k += blockDim.x) reinterpret_cast<unsigned*>(sL)[k] = a[k];
+  for (int k = threadIdx.x; k < nb; k += blockDim.x) reinterpret_cast<unsigned*>(sX)[k] = b[k];
+}
+constexpr int TEAM_LEVELS = 24;
+
+// one cluster (of 1 to CLUSTER_MAX blocks)
+template <typename T, int FORM, int MODEL>
+__global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail(const Level<T>* __restrict__ Ls, const Xfer<T>* __restrict__ Xs,
+                                                       int l0, int nl, int tail_start, int handoff, Phys<T> P, int nu1,
+                                                       int nu2, int cmax, T crtol, int gamma, int gamma_levels,
+                                                       unsigned long long* stats, int ordering) {
+  __shared__ ClusterShared sh;
+  __shared__ Level<T> sL[TEAM_LEVELS];
+  __shared__ Xfer<T> sX[TEAM_LEVELS];
+  stage_levels(Ls, Xs, l0, nl, sL, sX);
+  ClusterTeam tm(&sh);
+  tm.sync();
+  unsigned long long updates = 0;
+  team_cycle<T, FORM, MODEL>(GridLevels<T>{sL, sX, l0, tail_start}, l0, nl, P, nu1, nu2, cmax, crtol, gamma,
+                             gamma_levels, updates, ordering, handoff, tm);
+  if (threadIdx.x == 0 && tm.lead() && stats) atomicAdd(stats, updates);
+  tm.sync();                           // (no block leaves while another may still write to its shared memory)
+}
+
+// The coarse levels of a big grid as one cooperative launch, a grid barrier
+// between phases instead of a launch per stage; block 0 alone takes the
+// single-block tail's levels.  slots: three global words for the grid
+// reductions; stats: the update count
 template <typename T, int FORM, int MODEL>
 __global__ void __launch_bounds__(COOP_THREADS) k_coop_cycle(const Level<T>* __restrict__ Ls,
                                                              const Xfer<T>* __restrict__ Xs, int l0, int nl,
@@ -732,14 +826,12 @@ __global__ void __launch_bounds__(COOP_THREADS) k_coop_cycle(const Level<T>* __r
                                                              T crtol, int gamma, int gamma_levels,
                                                              unsigned long long* stats, unsigned long long* slots) {
   __shared__ unsigned long long sm[33];
-  GridTeam tm{slots, 0};
+  GridTeam tm{slots, sm, 0, false};
   if (tm.rank() == 0) slots[0] = slots[1] = slots[2] = 0ull;
   tm.sync();
   unsigned long long updates = 0;
-  const DeviceLevels<T> tail{Ls, Xs};
-  block_cycle<T, FORM, MODEL, CoopLevels<T>, GridTeam, DeviceLevels<T>>(CoopLevels<T>{Ls, Xs, tail_start}, l0, nl, P,
-                                                                        nu1, nu2, cmax, crtol, gamma, gamma_levels,
-                                                                        sm, updates, 1, &tm, tail_start, &tail);
+  team_cycle<T, FORM, MODEL>(GridLevels<T>{Ls + l0, Xs + l0, l0, tail_start}, l0, nl, P, nu1, nu2, cmax, crtol, gamma,
+                             gamma_levels, updates, 1, tail_start, tm);
   if (tm.rank() == 0 && stats) atomicAdd(stats, updates);
 }
 
@@ -768,6 +860,34 @@ inline Launch3 launch3(int nx, int n1, int n2, int bx_force = 0) {
   L.block = dim3(bx, 1, 1);
   L.grid = dim3((nx + bx - 1) / bx, n1, n2);
   return L;
+}
+
+// launches `clusters` clusters of `blocks` thread blocks; clusters of more
+// than 8 blocks need the kernel's consent (a non-portable size), and a device
+// that cannot place such a cluster takes the next smaller power of two
+template <typename... KA, typename... A>
+inline cudaError_t launch_cluster(void (*kern)(KA...), int blocks, int clusters, int threads, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  if (blocks > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    blocks = 8;
+  }
+  for (;; blocks >>= 1) {
+    at.val.clusterDim.x = blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(blocks * clusters);
+    if (blocks <= 8) break;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) break;
+    cudaGetLastError();
+  }
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<KA>(args)...);
 }
 
 // host: calls fn(LawTag<model>{}) for a runtime law (COMPOSITE included)
@@ -923,12 +1043,14 @@ struct Dispatch {
     });
     return e;
   }
-  static void tail(const Level<T>* dLs, const Xfer<T>* dXs, int l0, int nl, const Phys<T>& P, int model,
-                   int nu1, int nu2, int cmax, T crtol, int gamma, int gamma_levels, unsigned long long* stats,
-                   int ordering, cudaStream_t s) {
+  // one cluster of `blocks` blocks (a power of two up to CLUSTER_MAX; fewer
+  // when the device cannot place that many)
+  static void tail(const Level<T>* dLs, const Xfer<T>* dXs, int l0, int nl, const TeamShape& ts, const Phys<T>& P,
+                   int model, int nu1, int nu2, int cmax, T crtol, int gamma, int gamma_levels,
+                   unsigned long long* stats, int ordering, cudaStream_t s) {
     by_model(model, [&](auto m) {
-      k_tail<T, FORM, decltype(m)::value><<<1, TAIL_THREADS, 0, s>>>(dLs, dXs, l0, nl, P, nu1, nu2, cmax, crtol,
-                                                                      gamma, gamma_levels, stats, ordering);
+      launch_cluster(k_tail<T, FORM, decltype(m)::value>, ts.blocks, 1, TAIL_THREADS, s, dLs, dXs, l0, nl,
+                     ts.tail_start, ts.handoff, P, nu1, nu2, cmax, crtol, gamma, gamma_levels, stats, ordering);
     });
   }
 };

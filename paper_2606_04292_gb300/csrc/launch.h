@@ -25,6 +25,43 @@ struct Geom {
   double Lv;            // length of the vertical axis
 };
 
+// How the coarse tail runs: one cluster of `blocks` blocks; levels from
+// `handoff` on by its first block alone; transfers below `tail_start` as the
+// grid kernels take them (nested formulas), from it on through the tables.
+struct TeamShape {
+  int blocks, handoff, tail_start;
+};
+
+// The shape for levels l0 .. nl - 1 of `cells` cells each.  A phase of a
+// small level takes one point update's latency wherever it runs, so a level
+// goes to one block once a block's barrier beats the cluster's: at 256 cells
+// in FP64 (solo below 64: two steps of the 128-cell column 2.94 ms, 256: 2.74)
+// and 1024 in FP32 (256: Gardner 128^2 3.74 ms, 1024: 3.62).  Blocks: one per
+// 128 (FP64) or 256 (FP32) cells, half and twice that within 2%.
+template <typename T>
+inline TeamShape team_shape(const long long* cells, int l0, int nl, int tail_start) {
+  const long long solo = sizeof(T) == 8 ? 256 : 1024, per = sizeof(T) == 8 ? 128 : 256;
+  TeamShape ts{1, l0, tail_start};
+  if (cells[l0] <= solo) return ts;
+  while (ts.blocks < 16 && ts.blocks * per < cells[l0]) ts.blocks *= 2;
+  ts.handoff = nl;
+  for (int l = l0; l < nl; ++l)
+    if (cells[l] <= solo) { ts.handoff = l; break; }
+  return ts;
+}
+
+// The biggest level (cells) a cycle runs in the tail's cluster instead of as a
+// launch per stage: where 16 SMs still finish a phase in less than a launch
+// (~5 us in a graph).  FP64: 65^2 in (257^2 strip 3.08 -> 2.92 ms), 24^3 out
+// (96^3 21.0 -> 21.6 ms with it).  FP32: 2-d levels to 128^2 (two-layer 256^2
+// 15.8 -> 14.5 ms), 3-d ones only to 16384 cells (32^3: 256^3 step 1.5% slower
+// with it).  Batched contexts: 33^3 too, so that the mix leaves its grid
+// stages together (8 requests 9.1 -> 7.6 ms).
+template <typename T>
+inline long long cluster_cells(int dim, bool batched = false) {
+  return sizeof(T) == 8 ? 4608 : batched ? 66000 : dim < 3 ? 32768 : 16384;
+}
+
 // FP64, psi as unknown
 void sweep64(const Level<double>& L, const Phys<double>& P, int model, int color, cudaStream_t s);
 void residual64(const Level<double>& L, const Phys<double>& P, int model, unsigned long long* norm,
@@ -34,8 +71,8 @@ void restrict64(const Level<double>& F, const Level<double>& C, const Xfer<doubl
                 const double* fb, double* ca, double* cb, cudaStream_t s);
 void prolong64(const Level<double>& F, const Level<double>& C, const Xfer<double>& X, cudaStream_t s);
 // ordering: 1 red-black, 0 lexicographic (hyperplane by hyperplane)
-void tail64(const Level<double>* dLs, const Xfer<double>* dXs, int l0, int nl, const Phys<double>& P,
-            int model, int nu1, int nu2, int cmax, double crtol, int gamma, int gamma_levels,
+void tail64(const Level<double>* dLs, const Xfer<double>* dXs, int l0, int nl, const TeamShape& ts,
+            const Phys<double>& P, int model, int nu1, int nu2, int cmax, double crtol, int gamma, int gamma_levels,
             unsigned long long* stats, int ordering, cudaStream_t s);
 // one lexicographic NGS sweep (a launch per hyperplane i0 + i1 + i2 = const)
 void sweep_lex64(const Level<double>& L, const Phys<double>& P, int model, cudaStream_t s);
@@ -52,8 +89,8 @@ void tau32(const Level<float>& C, const Phys<float>& P, int model, cudaStream_t 
 void restrict32(const Level<float>& F, const Level<float>& C, const Xfer<float>& X, const float* fa,
                 const float* fb, float* ca, float* cb, cudaStream_t s, int cs_mask = 0);
 void prolong32(const Level<float>& F, const Level<float>& C, const Xfer<float>& X, cudaStream_t s);
-void tail32(const Level<float>* dLs, const Xfer<float>* dXs, int l0, int nl, const Phys<float>& P,
-            int model, int nu1, int nu2, int cmax, float crtol, int gamma, int gamma_levels,
+void tail32(const Level<float>* dLs, const Xfer<float>* dXs, int l0, int nl, const TeamShape& ts,
+            const Phys<float>& P, int model, int nu1, int nu2, int cmax, float crtol, int gamma, int gamma_levels,
             unsigned long long* stats, int ordering, cudaStream_t s);
 void sweep_lex32(const Level<float>& L, const Phys<float>& P, int model, cudaStream_t s);
 // the cycle from level l0 down as one cooperative launch of `blocks` blocks
@@ -157,6 +194,7 @@ struct BJob32 {
   const Level<float>* dLs;           // the context's device level views (coarse tail)
   const Xfer<float>* dXs;
   int level, nlev;
+  int tail_start, handoff;           // TeamShape of the coarse tail from this level
   int model;                         // the context's law (HAVERKAMP, GARDNER, VANGENUCHTEN, COMPOSITE)
   unsigned long long* norm;          // the context's inner-norm slot (float bits)
   unsigned long long* stats;         // the context's coarse-tail update counter
@@ -177,8 +215,8 @@ int batch_blocks(int op, const BJob32& j);
 // P.newton_k; color for BOP_SWEEP; with_norm: the defect's max into each
 // descriptor's norm slot (BOP_RESID)
 void batch32(int op, int nk, const BJob32* table, const BList& list, int color, bool with_norm, cudaStream_t s);
-// the coarse tail from each listed descriptor's level: one block each
-void batch_tail32(const BJob32* table, const BList& list, int nu1, int nu2, int cmax, float crtol, int gamma,
+// the coarse tail from each listed descriptor's level: a cluster of `blocks` blocks each
+void batch_tail32(const BJob32* table, const BList& list, int blocks, int nu1, int nu2, int cmax, float crtol, int gamma,
                   int gamma_levels, cudaStream_t s);
 
 }  // namespace rich

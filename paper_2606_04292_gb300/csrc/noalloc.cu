@@ -9,9 +9,9 @@
 // step needs (multigrid hierarchy, coefficients, transfer tables, norms)
 // lives in one fixed array in the library's own device memory.
 //
-// The whole step runs in one thread block (a variant of the coarse-tail
-// kernel that also does the per-step preparation and the stop loop), so the
-// grid is limited to RICHARDS_NOALLOC_MAX_CELLS cells.
+// The whole step runs in one cluster of thread blocks (a variant of the
+// coarse-tail kernel that also does the per-step preparation and the stop
+// loop), so the grid is limited to RICHARDS_NOALLOC_MAX_CELLS cells.
 #include <cmath>
 #include <cstring>
 
@@ -41,6 +41,7 @@ struct NaLevel {
 
 struct NaPlan {
   int nlev, dim, model, scheme, max_cycles, nu1, nu2, cmax, gamma, gamma_levels, ordering;
+  int blocks, handoff;             // the team: blocks of its cluster, first level one block runs alone
   int ctx_mode;                    // 1: a context's hierarchy (its transfer tables, soil and sink arrays)
   double crtol, tol, dt, Lv, h[3];
   double slo[3], shi[3];           // prolongation ghost factors per axis
@@ -57,17 +58,18 @@ struct NaPlan {
 // ---------------------------------------------------------------------------
 // device pieces
 // ---------------------------------------------------------------------------
-// transfer tables of every level, built by the block
-// (*overflow is set when a coarse cell would take more than RMAX fine
-// contributors along an axis; ceil(n/2) coarsening gives at most 4)
-__device__ void na_tables(const NaPlan& p, int* overflow) {
+// transfer tables of every level, built by the team (returns whether a
+// coarse cell would take more than RMAX fine contributors along an axis;
+// ceil(n/2) coarsening gives at most 4)
+__device__ bool na_tables(const NaPlan& p, ClusterTeam& tm) {
+  unsigned long long overflow = 0;
   for (int l = 0; l + 1 < p.nlev; ++l) {
     const NaLevel& F = p.lev[l];
     const NaLevel& C = p.lev[l + 1];
     const int nfa[3] = {F.L.n0, F.L.n1, F.L.n2}, nca[3] = {C.L.n0, C.L.n1, C.L.n2};
     for (int ax = 0; ax < 3; ++ax) {
       const int nf = nfa[ax], nc = nca[ax];
-      for (int i = threadIdx.x; i < nf; i += blockDim.x) {
+      for (int i = tm.rank(); i < nf; i += tm.size()) {
         int idx[2];
         double w[2];
         int cnt;
@@ -78,7 +80,7 @@ __device__ void na_tables(const NaPlan& p, int* overflow) {
           F.pw[ax][2 * i + k] = k < cnt ? w[k] : 0.0;
         }
       }
-      for (int J = threadIdx.x; J < nc; J += blockDim.x) {
+      for (int J = tm.rank(); J < nc; J += tm.size()) {
         int cnt = 0;
         double s = 0.0;
         const int lo = nf == 1 ? 0 : (2 * J - 4 > 0 ? 2 * J - 4 : 0);
@@ -90,7 +92,7 @@ __device__ void na_tables(const NaPlan& p, int* overflow) {
           interp_row(nf, nc, i, 1.0, 1.0, idx, w, c2);
           for (int k = 0; k < c2; ++k)
             if (idx[k] == J) {
-              if (cnt == RMAX) { *overflow = 1; continue; }
+              if (cnt == RMAX) { overflow = 1; continue; }
               F.ri[ax][RMAX * J + cnt] = i;
               F.rw[ax][RMAX * J + cnt] = w[k];
               ++cnt;
@@ -102,16 +104,16 @@ __device__ void na_tables(const NaPlan& p, int* overflow) {
       }
     }
   }
-  __syncthreads();
+  return tm.max(overflow) != 0;
 }
 
 // lagged state, Kc, history and the right side of the finest level
 template <int MODEL>
-__device__ void na_prepare(const NaPlan& p) {
+__device__ void na_prepare(const NaPlan& p, ClusterTeam& tm) {
   const NaLevel& F = p.lev[0];
   const Level<double>& L = F.L;
   const Phys<double>& P = p.P;
-  for (long long i = threadIdx.x; i < L.ncell; i += blockDim.x) {
+  for (long long i = tm.rank(); i < L.ncell; i += tm.size()) {
     const double p1 = p.p1_field ? p.p1_field[i] : P.p1, p2 = p.p2_field ? p.p2_field[i] : P.p2;
     if (!p.ctx_mode) {
       if (F.p1w) F.p1w[i] = p1;
@@ -151,11 +153,11 @@ __device__ void na_prepare(const NaPlan& p) {
       F.smaxw[i] = depth <= D ? p.Tp * exp(-depth / lam) / Z : 0.0;
     }
   }
-  __syncthreads();
+  tm.sync();
   const int v = p.dim - 1;
   const int nn[3] = {L.n0, L.n1, L.n2};
   const long long stride[3] = {1, L.n0, (long long)L.n0 * L.n1};
-  for (long long i = threadIdx.x; i < L.ncell; i += blockDim.x) {
+  for (long long i = tm.rank(); i < L.ncell; i += tm.size()) {
     int ii[3];
     cell_coords(L.n0, L.n1, i, ii[0], ii[1], ii[2]);
     double gi = L.g[i];
@@ -192,12 +194,12 @@ __device__ void na_prepare(const NaPlan& p) {
       }
     L.g[i] = gi;
   }
-  __syncthreads();
+  tm.sync();
   // coarse coefficients: restricted Kc, soil parameters, sink, face conductances
   for (int l = 0; l + 1 < p.nlev; ++l) {
     const NaLevel& Fl = p.lev[l];
     const NaLevel& Cl = p.lev[l + 1];
-    for (long long J = threadIdx.x; J < Cl.L.ncell; J += blockDim.x) {
+    for (long long J = tm.rank(); J < Cl.L.ncell; J += tm.size()) {
       int J0, J1, J2;
       cell_coords(Cl.L.n0, Cl.L.n1, J, J0, J1, J2);
       Cl.Kcw[J] = restrict_at(Fl.L, Fl.X, Fl.L.Kc, J0, J1, J2);
@@ -213,7 +215,7 @@ __device__ void na_prepare(const NaPlan& p) {
       for (int a = 0; a < 3; ++a)
         if (a != ax) oa[k++] = a;
       const long long nc = (long long)nC[oa[0]] * nC[oa[1]];
-      for (long long J = threadIdx.x; J < nc; J += blockDim.x) {
+      for (long long J = tm.rank(); J < nc; J += tm.size()) {
         const int J0 = (int)(J % nC[oa[0]]), J1 = (int)(J / nC[oa[0]]);
         double s = 0.0;
         for (int a1 = 0; a1 < Fl.X.rc[oa[1]][J1]; ++a1)
@@ -223,20 +225,16 @@ __device__ void na_prepare(const NaPlan& p) {
         Cl.kbw[f][J] = s;
       }
     }
-    __syncthreads();
+    tm.sync();
   }
 }
 
 struct PlanLevels {
   const NaLevel* lev;
   __device__ const Level<double>& L(int l) const { return lev[l].L; }
-  __device__ double restrict(int l, const double* fine, int J0, int J1, int J2) const {
-    return restrict_at(lev[l].L, lev[l].X, fine, J0, J1, J2);
-  }
   __device__ void restrict2(int l, const double* fa, const double* fb, int J0, int J1, int J2, double& a,
                             double& b) const {
-    a = restrict(l, fa, J0, J1, J2);
-    b = restrict(l, fb, J0, J1, J2);
+    restrict2_at(lev[l].L, lev[l].X, fa, fb, J0, J1, J2, a, b);
   }
   __device__ double prolong(int l, int i0, int i1, int i2) const {
     return prolong_at(lev[l + 1].L, lev[l].X, i0, i1, i2);
@@ -244,43 +242,44 @@ struct PlanLevels {
 };
 
 template <int MODEL>
-__global__ void __launch_bounds__(TAIL_THREADS) k_small_step(const __grid_constant__ NaPlan p) {
-  __shared__ unsigned long long sm[33];
-  __shared__ int overflow;
-  if (threadIdx.x == 0) overflow = 0;
-  __syncthreads();
-  if (!p.ctx_mode) na_tables(p, &overflow);   // ends with a barrier
-  if (overflow) {                   // (uniform over the block)
-    if (threadIdx.x == 0) {
+__global__ void __launch_bounds__(TAIL_THREADS, 1) k_small_step(const __grid_constant__ NaPlan p) {
+  __shared__ ClusterShared sh;
+  ClusterTeam tm(&sh);
+  tm.sync();
+  const bool first = threadIdx.x == 0 && tm.lead();
+  if (!p.ctx_mode && na_tables(p, tm)) {
+    if (first) {
       p.stats[0] = 0.0;
       p.stats[1] = p.stats[2] = 0.0;
       p.stats[3] = (double)RICH_EINVAL;
       p.stats[4] = 0.0;
     }
-    return;
+    return;                         // (na_tables ends with a barrier of the team)
   }
-  na_prepare<MODEL>(p);
+  na_prepare<MODEL>(p, tm);
   const Phys<double>& P = p.P;
   const double teff = 1.0 / P.a;
-  double r = teff * block_defect_norm<double, FORM_DIRECT, MODEL>(p.lev[0].L, P, sm);
-  const double r0 = r;
+  double r = 0.0, r0 = 0.0;
   int cycles = 0;
   unsigned long long updates = 0;
-  while (!(r <= p.tol) && cycles < p.max_cycles && !isnan(r)) {
-    block_cycle<double, FORM_DIRECT, MODEL>(PlanLevels{p.lev}, 0, p.nlev, P, p.nu1, p.nu2, p.cmax, p.crtol, p.gamma,
-                                            p.gamma_levels, sm, updates, p.ordering);
+  for (;;) {
+    r = teff * team_defect<double, FORM_DIRECT, MODEL>(p.lev[0].L, P, false, tm);
+    if (cycles == 0) r0 = r;
+    if (r <= p.tol || cycles >= p.max_cycles || isnan(r)) break;
+    team_cycle<double, FORM_DIRECT, MODEL>(PlanLevels{p.lev}, 0, p.nlev, P, p.nu1, p.nu2, p.cmax, p.crtol, p.gamma,
+                                           p.gamma_levels, updates, p.ordering, p.handoff, tm);
     ++cycles;
-    r = teff * block_defect_norm<double, FORM_DIRECT, MODEL>(p.lev[0].L, P, sm);
   }
   const Level<double>& F = p.lev[0].L;
-  for (long long i = threadIdx.x; i < F.ncell; i += blockDim.x) p.psi_out[i] = F.u[i];
-  if (threadIdx.x == 0) {
+  for (long long i = tm.rank(); i < F.ncell; i += tm.size()) p.psi_out[i] = F.u[i];
+  if (first) {
     p.stats[0] = cycles;
     p.stats[1] = r0;
     p.stats[2] = r;
     p.stats[3] = isnan(r) ? (double)RICH_ENAN : (r <= p.tol ? (double)RICH_OK : (double)RICH_ENOCONV);
     p.stats[4] = (double)updates;
   }
+  tm.sync();                        // (no block leaves while another may still write to its shared memory)
 }
 
 // Lays out the hierarchy of a small step over `base` (capacity doubles; base
@@ -412,14 +411,18 @@ long long build_plan(const richards_grid* grid, const richards_soil* soil, const
   P.sink = sink->enabled;
   P.lag = o.bdf2_lag;
   if (cx) P.mats = cx->mats;
+  long long cells[NA_MAXLEV];
+  for (int l = 0; l < nlev; ++l) cells[l] = p.lev[l].L.ncell;
+  const TeamShape ts = team_shape<double>(cells, 0, nlev, nlev);
+  p.blocks = ts.blocks;
+  p.handoff = ts.handoff;
   return used;
 }
 
 void launch_plan(const NaPlan& p, cudaStream_t s) {
-  if (p.model == RICH_HAVERKAMP) k_small_step<HAVERKAMP><<<1, TAIL_THREADS, 0, s>>>(p);
-  else if (p.model == RICH_GARDNER) k_small_step<GARDNER><<<1, TAIL_THREADS, 0, s>>>(p);
-  else if (p.model == COMPOSITE) k_small_step<COMPOSITE><<<1, TAIL_THREADS, 0, s>>>(p);
-  else k_small_step<VANGENUCHTEN><<<1, TAIL_THREADS, 0, s>>>(p);
+  by_model(p.model, [&](auto m) {
+    launch_cluster(k_small_step<decltype(m)::value>, p.blocks, 1, TAIL_THREADS, s, p);
+  });
 }
 
 // device address of the scratch array, looked up once per device
