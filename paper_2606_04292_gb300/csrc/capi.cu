@@ -85,6 +85,7 @@ struct richards_ctx {
   int team_start64 = 0, team_start32 = 0, team_start_batch = 0;
   HLevel L[MAXLEV];
   richards_soil soil{};
+  rich::fl::Prep law_q{};        // the uniform soil's powers in fixed point
   bool soil_set = false, het_p1 = false, het_p2 = false, het_Ks = false;
   // layered soil (richards_set_materials): soil.model is then rich::COMPOSITE
   bool layered = false;
@@ -488,9 +489,12 @@ Phys<T> phys(const richards_ctx* c) {
   P.tr = (T)c->soil.theta_r;
   P.p1 = (T)c->soil.p1; P.p2 = (T)c->soil.p2; P.p3 = (T)c->soil.p3; P.p4 = (T)c->soil.p4;
   P.h1 = (T)c->sink.h1; P.h2 = (T)c->sink.h2; P.h3 = (T)c->sink.h3; P.h4 = (T)c->sink.h4;
+  rich::set_sink_slopes(P);
   P.newton_k = c->opts.newton_iters;
   P.sink = c->sink.enabled;
   P.lag = c->opts.bdf2_lag;
+  if constexpr (std::is_same<T, double>::value)
+    if (!c->layered) P.q = c->law_q;
   if (c->layered) {
     if constexpr (std::is_same<T, double>::value) P.mats = c->dmat64;
     else P.mats = c->dmat32;
@@ -930,28 +934,29 @@ richards_status run_inner_loop(richards_ctx* c, double target, int* cycles) {
   return RICH_OK;
 }
 
+// blocks of the set-up cluster: one below 2048 cells (faces: of the finest
+// level's boundary; else of the first level it restricts)
+int setup_blocks(const richards_ctx* c, bool faces) {
+  long long work = c->L[c->opts.precision >= 1 ? c->team_start32 : c->team_start64].ncell;
+  for (int f = 0; faces && f < 2 * c->grid.dim; ++f) work += c->L[0].nface[f];
+  return work <= 2048 ? 1 : rich::CLUSTER_MAX;
+}
+
 // coarse copies of the lagged conductivity and boundary conductances
 // (mixed mode: the coarse coefficients only feed the FP32 inner cycles, so
 // they are restricted in FP32 from the finest level's FP32 copies)
 richards_status restrict_coefficients(richards_ctx* c) {
   Prof pr(c, "coefficients", 0, c->L[0].ncell);
   if (c->opts.precision >= 1) {
-    for (int f = 0; f < 2 * c->grid.dim; ++f) rich::to_float(c->L[0].kb[f], c->L[0].kbf[f], c->L[0].nface[f], c->s);
-    for (int l = 0; l + 1 < c->nlev; ++l) {
-      const Level<float> F = view32(c, l), C = view32(c, l + 1);
-      rich::restrict32(F, C, xfer32(c, l), c->L[l].Kcf, nullptr, c->L[l + 1].Kcf, nullptr, c->s);
-      for (int f = 0; f < 2 * c->grid.dim; ++f)
-        rich::restrict_face32(geom(c, l), geom(c, l + 1), xfer32(c, l), f / 2, c->L[l].kbf[f], c->L[l + 1].kbf[f],
-                              c->s);
-    }
+    for (int l = 0; l < c->team_start32 && l + 1 < c->nlev; ++l)
+      rich::restrict32(view32(c, l), view32(c, l + 1), xfer32(c, l), c->L[l].Kcf, nullptr, c->L[l + 1].Kcf, nullptr,
+                       c->s);
+    rich::team_setup32(c->dL32, c->dX32, c->nlev, c->team_start32, setup_blocks(c, true), false, c->L[0].kb, c->s);
     return check_launch(c);
   }
-  for (int l = 0; l + 1 < c->nlev; ++l) {
-    const Level<double> F = view64(c, l), C = view64(c, l + 1);
-    rich::restrict64(F, C, xfer64(c, l), c->L[l].Kc, nullptr, c->L[l + 1].Kc, nullptr, c->s);
-    for (int f = 0; f < 2 * c->grid.dim; ++f)
-      rich::restrict_face64(geom(c, l), geom(c, l + 1), xfer64(c, l), f / 2, c->L[l].kb[f], c->L[l + 1].kb[f], c->s);
-  }
+  for (int l = 0; l < c->team_start64 && l + 1 < c->nlev; ++l)
+    rich::restrict64(view64(c, l), view64(c, l + 1), xfer64(c, l), c->L[l].Kc, nullptr, c->L[l + 1].Kc, nullptr, c->s);
+  rich::team_setup64(c->dL64, c->dX64, c->nlev, c->team_start64, setup_blocks(c, true), c->s);
   return check_launch(c);
 }
 
@@ -1226,11 +1231,15 @@ richards_status defect_from_g(richards_ctx* c) {
 
 // the coarse copies of the inner problem's frozen state psi0
 void restrict_psi0(richards_ctx* c) {
-  for (int l = 0; l + 1 < c->nlev; ++l) {
+  const int ts = c->team_start32;
+  for (int l = 0; l < ts && l + 1 < c->nlev; ++l) {
     Prof pr(c, "restrict_psi0", l, c->L[l + 1].ncell);
     rich::restrict32(view32(c, l), view32(c, l + 1), xfer32(c, l), c->L[l].psi0f, nullptr, c->L[l + 1].psi0f,
                      nullptr, c->s, c->L[l].cs ? 1 : 0);
   }
+  if (ts + 1 >= c->nlev) return;
+  Prof pr(c, "restrict_psi0", ts, c->L[ts].ncell);
+  rich::team_setup32(c->dL32, c->dX32, c->nlev, ts, setup_blocks(c, false), true, nullptr, c->s);
 }
 
 richards_status step_mixed(richards_ctx* c, richards_step_info* info) {
@@ -1943,6 +1952,7 @@ richards_status richards_set_soil(richards_ctx* c, const richards_soil* s) {
     for (long long i = 0; i < N; ++i)
       if (!(s->p2_field[i] > 1.0)) return fail(c, RICH_EINVAL, "van Genuchten n field must exceed 1");
   c->soil = *s;
+  c->law_q = rich::law_prep(s->model, s->p1, s->p2);
   c->soil.Ks_field = c->soil.p1_field = c->soil.p2_field = nullptr;
   c->layered = false;
   c->nmat = 0;
@@ -2074,7 +2084,7 @@ richards_status richards_set_materials(richards_ctx* c, const richards_material*
   rich::DDMat tdd[rich::MAXMAT] = {};
   for (int m = 0; m < nmat; ++m) {
     const richards_material& M = mats[m];
-    t64[m] = rich::MatLaw<double>{M.model, M.theta_s, M.theta_r, M.p3, M.p4};
+    t64[m] = rich::MatLaw<double>{M.model, M.theta_s, M.theta_r, M.p3, M.p4, rich::law_prep(M.model, M.p1, M.p2)};
     t32[m] = rich::MatLaw<float>{M.model, (float)M.theta_s, (float)M.theta_r, (float)M.p3, (float)M.p4};
     tdd[m] = rich::make_ddmat(t64[m]);
   }

@@ -198,12 +198,14 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
   P64.p1 = D.p1; P64.p2 = D.p2; P64.p3 = D.p3; P64.p4 = D.p4;
   P64.h1 = A.h1; P64.h2 = A.h2; P64.h3 = A.h3; P64.h4 = A.h4;
   P64.newton_k = A.newton_k; P64.sink = A.sink; P64.lag = A.lag;
+  set_sink_slopes(P64);
   if (threadIdx.x == 0) {              // (read after the barriers of the step's preparation)
     Phys<float> P32{};
     P32.xi = (float)A.xi; P32.kappa = (float)A.kappa; P32.ts = (float)D.ts; P32.tr = (float)D.tr;
     P32.p1 = (float)D.p1; P32.p2 = (float)D.p2; P32.p3 = (float)D.p3; P32.p4 = (float)D.p4;
     P32.h1 = (float)A.h1; P32.h2 = (float)A.h2; P32.h3 = (float)A.h3; P32.h4 = (float)A.h4;
     P32.newton_k = A.newton_k; P32.sink = A.sink; P32.lag = A.lag;
+    set_sink_slopes(P32);
     S->P = P32;
     S->nu1 = A.nu1; S->nu2 = A.nu2; S->cmax = A.cmax; S->gamma = A.gamma; S->gamma_levels = A.gamma_levels;
     S->inner_cycles = A.inner_cycles;

@@ -86,11 +86,24 @@ struct MatLaw {
   int model;
   T ts, tr, p3, p4;
 };
+template <>
+struct MatLaw<double> {
+  int model;
+  double ts, tr, p3, p4;
+  fl::Prep q;                    // the law's powers, prepared (Gardner: n = 1, alpha = 1)
+};
 
 struct DDMat;                    // float-float copy of a MatLaw (ddmath.cuh)
 
 template <typename T>
-struct Phys {
+struct UniformLaw {};
+template <>
+struct UniformLaw<double> {
+  fl::Prep q;                    // a uniform soil's powers, prepared
+};
+
+template <typename T>
+struct Phys : UniformLaw<T> {
   T a, xi, kappa;
   T ts, tr;                      // theta_s, theta_r
   T p1, p2, p3, p4;              // scalar soil parameters
@@ -98,12 +111,24 @@ struct Phys {
   int newton_k;                  // > 0: fixed steps; 0: to round-off
   int sink;
   int lag;                       // BDF2: 1 lags K and the xi term at psi^n, 0 at 2 psi^n - psi^(n-1)
+  T r12, r34;                    // 1/(h1 - h2), 1/(h3 - h4)
   const MatLaw<T> *mats;         // COMPOSITE: material table (device, MAXMAT entries at most)
   const DDMat *ddmats;           // COMPOSITE, float-float outer layer: the same table as pairs
 };
 
 template <int M>
 using LawTag = std::integral_constant<int, M>;
+
+// a law's powers prepared on the host (fixlaw.cuh)
+inline fl::Prep law_prep(int model, double p1, double p2) {
+  return model == GARDNER ? fl::host_prep(false, 1.0, 1.0) : fl::host_prep(model == VANGENUCHTEN, p1, p2);
+}
+// the sink's slopes
+template <typename T>
+__host__ __device__ __forceinline__ void set_sink_slopes(Phys<T>& P) {
+  P.r12 = P.h1 != P.h2 ? T(1) / (P.h1 - P.h2) : T(0);
+  P.r34 = P.h3 != P.h4 ? T(1) / (P.h3 - P.h4) : T(0);
+}
 
 // Calls fn(LawTag<law>{}, phys) with the law of a cell and the physics
 // record that carries its theta_s, theta_r, p3, p4: MODEL and P themselves,
@@ -203,13 +228,19 @@ __device__ __forceinline__ bool unsaturated(double psi) {
   return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
 }
 
-// A cell's law with its parameters prepared once per point solve.
+// A cell's law with its parameters prepared once per point solve (uniform
+// soils: once per launch, P.q; layered soils: once per material).
 template <int MODEL>
 struct LawCell {
   fl::Prep q;
   double p1, p2, ds, cs;      // cs: the factor of d theta/d psi (ds beta, ds alpha, ds (n - 1))
-  __device__ __forceinline__ LawCell(double a, double b, const Phys<double>& P) : p1(a), p2(b), ds(P.ts - P.tr) {
-    if (MODEL != GARDNER) q = fl::prep<MODEL == VANGENUCHTEN>(a, b);
+  // uniform: P.q is this cell's
+  __device__ __forceinline__ LawCell(double a, double b, bool uniform, const Phys<double>& P)
+      : p1(a), p2(b), ds(P.ts - P.tr) {
+    if (MODEL != GARDNER) {
+      if (uniform) q = P.q;
+      else q = fl::prep<MODEL == VANGENUCHTEN>(a, b);
+    }
     cs = ds * (MODEL == GARDNER ? a : (MODEL == HAVERKAMP ? b : b - 1.0));
   }
   // theta(psi) and theta'(psi)
@@ -234,6 +265,50 @@ struct LawCell {
   }
 };
 
+// (the increment form prepares nothing here)
+template <>
+struct LawCell<-1> {};
+
+static __device__ __noinline__ double2 slow_se_any(int law, double h, double p1, double p2) {
+  if (law == HAVERKAMP) return slow_se_slope<HAVERKAMP>(h, p1, p2);
+  if (law == GARDNER) return slow_se_slope<GARDNER>(h, p1, p2);
+  return slow_se_slope<VANGENUCHTEN>(h, p1, p2);
+}
+
+// Layered soils: every lane its own material's law, in one instruction stream.
+template <>
+struct LawCell<COMPOSITE> {
+  fl::Prep q;
+  int law;
+  double p1, p2, ds, cs;
+  __device__ __forceinline__ LawCell(double a, double b, unsigned m, const Phys<double>& P)
+      : p1(a), p2(b), ds(P.ts - P.tr) {
+    q = P.mats[m].q;
+    law = P.mats[m].model;
+    cs = ds * (law == GARDNER ? a : (law == HAVERKAMP ? b : b - 1.0));
+  }
+  template <bool SLOPE>
+  __device__ __forceinline__ void any(double psi, const Phys<double>& P, double& th, double& dth) const {
+    static_assert(HAVERKAMP == fl::ANY_HAVERKAMP && GARDNER == fl::ANY_GARDNER && VANGENUCHTEN == fl::ANY_VANGENUCHTEN,
+                  "law numbers");
+    if (!unsaturated(psi)) { th = P.ts; dth = 0.0; return; }
+    const unsigned long long hb = fl::dbits(psi) ^ 0x8000000000000000ull;
+    bool ok = q.ok;
+    double Se, s = 0.0;
+    fl::se_any<SLOPE>(law, q, p1, hb, ok, Se, s);
+    if (!ok) {
+      const double2 v = slow_se_any(law, -psi, p1, p2);
+      Se = v.x;
+      s = v.y;
+    }
+    th = P.tr + ds * Se;
+    if (SLOPE) dth = cs * s;
+  }
+  __device__ __forceinline__ void eval(double psi, const Phys<double>& P, double& th, double& dth) const {
+    any<true>(psi, P, th, dth);
+  }
+};
+
 template <int MODEL>
 __device__ __forceinline__ double theta_only_d(double psi, double p1, double p2, const Phys<double>& P) {
   if (!unsaturated(psi)) return P.ts;
@@ -242,6 +317,28 @@ __device__ __forceinline__ double theta_only_d(double psi, double p1, double p2,
   double Se = MODEL == GARDNER ? fl::exp_gardner(p1, hb, ok) : fl::se_only<MODEL == VANGENUCHTEN>(p1, p2, hb, ok);
   if (!ok) Se = slow_se<MODEL>(-psi, p1, p2);
   return P.tr + (P.ts - P.tr) * Se;
+}
+
+// theta at psi of a cell of a level (m: its material; uniform: no per-cell p1, p2)
+template <int MODEL>
+__device__ __forceinline__ double theta_cell(double psi, double p1, double p2, unsigned m, bool uniform,
+                                             const Phys<double>& P) {
+  if constexpr (MODEL == COMPOSITE) {
+    double th, dth;
+    Phys<double> Q = P;
+    Q.ts = P.mats[m].ts;
+    Q.tr = P.mats[m].tr;
+    LawCell<COMPOSITE>(p1, p2, m, Q).any<false>(psi, Q, th, dth);
+    return th;
+  } else {
+    if (MODEL == GARDNER || !uniform) return theta_only_d<MODEL>(psi, p1, p2, P);
+    if (!unsaturated(psi)) return P.ts;
+    const unsigned long long hb = fl::dbits(psi) ^ 0x8000000000000000ull;
+    bool ok = P.q.ok;
+    double Se = fl::se_prepared<MODEL == VANGENUCHTEN>(P.q, hb, ok);
+    if (!ok) Se = slow_se<MODEL>(-psi, p1, p2);
+    return P.tr + (P.ts - P.tr) * Se;
+  }
 }
 
 // Hydraulic conductivity.
@@ -448,9 +545,9 @@ template <typename T>
 __device__ __forceinline__ int feddes(T psi, const Phys<T>& P, T& a, T& da) {
   if (psi >= P.h1) { a = T(0); da = T(0); return 0; }
   if (psi < P.h4) { a = T(0); da = T(0); return 4; }
-  if (psi >= P.h2) { a = (P.h1 - psi) / (P.h1 - P.h2); da = T(-1) / (P.h1 - P.h2); return 1; }
+  if (psi >= P.h2) { a = (P.h1 - psi) * P.r12; da = -P.r12; return 1; }
   if (psi >= P.h3) { a = T(1); da = T(0); return 2; }
-  a = (psi - P.h4) / (P.h3 - P.h4); da = T(1) / (P.h3 - P.h4); return 3;
+  a = (psi - P.h4) * P.r34; da = P.r34; return 3;
 }
 
 template <typename T>
@@ -540,33 +637,26 @@ __device__ __forceinline__ double tol_of<double>() { return 1e-15; }
 template <>
 __device__ __forceinline__ float tol_of<float>() { return 1e-7f; }
 
-// Storage + sink part at x for either form (the defect's part of N).
+// Storage + sink part at x (the defect's part of N) of cell q of a level, of
+// material m.
 template <typename T, int FORM, int MODEL>
-__device__ __forceinline__ T storage(T x, T psi0, T p1, T p2, T smax, const Phys<T>& P) {
+__device__ __forceinline__ T storage(const Level<T>& L, T x, T psi0, T p1, T p2, T smax, unsigned m,
+                                     const Phys<T>& P) {
   if constexpr (FORM == FORM_DIRECT) {
     static_assert(sizeof(T) == 8, "direct form is FP64");
     double S, dS;
     sink_direct(x, smax, P, S, dS);
-    return P.a * theta_only_d<MODEL>(x, p1, p2, P) + S;
+    return P.a * theta_cell<MODEL>(x, p1, p2, m, !L.p1 && !L.p2, P) + S;
   } else {
     static_assert(sizeof(T) == 4, "increment form is FP32");
-    float Dth, dth, DS, dS;
-    dlaw_fast<MODEL>(psi0, x, p1, p2, P, Dth, dth);
-    sink_delta(psi0, x, smax, P, DS, dS);
-    return P.a * Dth + DS;
+    return with_law<MODEL>(P, m, [&](auto law, const Phys<T>& Q) {
+      float Dth, dth, DS, dS;
+      dlaw_fast<decltype(law)::value>(psi0, x, p1, p2, Q, Dth, dth);
+      sink_delta(psi0, x, smax, Q, DS, dS);
+      return Q.a * Dth + DS;
+    });
   }
 }
-
-// the FP64 law of a point solve (nothing to prepare in the increment form)
-template <int FORM, int MODEL>
-struct PointLaw {
-  template <typename T>
-  __device__ __forceinline__ PointLaw(T, T, const Phys<T>&) {}
-};
-template <int MODEL>
-struct PointLaw<FORM_DIRECT, MODEL> : LawCell<MODEL> {
-  __device__ __forceinline__ PointLaw(double p1, double p2, const Phys<double>& P) : LawCell<MODEL>(p1, p2, P) {}
-};
 
 // Scalar solve of  storage(x) + cc x = f  (eq. point-update).  The left side
 // increases strictly (cc > 0), the root lies in [lo, hi]; Newton from x0,
@@ -598,9 +688,10 @@ __device__ __forceinline__ double clamp_to(double x, double lo, double hi) {
   return less(x, lo) ? lo : (less(hi, x) ? hi : x);
 }
 
-template <typename T, int FORM, int MODEL, int NK = 0>
-__device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T smax,
-                                         const Phys<T>& P) {
+// SINK: 1 / 0 the physics have a sink / none, -1 as P.sink says.
+template <typename T, int FORM, int MODEL, int NK = 0, int SINK = -1>
+__device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T smax, const Phys<T>& P,
+                                         const LawCell<FORM == FORM_DIRECT ? MODEL : -1>& law) {
   if (!above_zero(cc)) {
     // no coupling and no shift (c = 0): shift kappa (x - x0), kappa = 1e-6 a,
     // which keeps the root and provides the bracket
@@ -608,6 +699,7 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
     f += (k - cc) * x0;
     cc = k;
   }
+  const bool has_sink = SINK != 0 && (SINK == 1 || P.sink) && smax > T(0);
   const T ds = P.ts - P.tr;
   T lo, hi;
   if constexpr (FORM == FORM_DIRECT) {
@@ -623,13 +715,12 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
   }
   T x = clamp_to(x0, lo, hi);
   const int maxit = NK > 0 ? NK : (P.newton_k > 0 ? P.newton_k : 200);
-  const PointLaw<FORM, MODEL> law(p1, p2, P);
   DBase B;
   T sa0 = T(0), sda0 = T(0);
   int sk0 = 0;
   if constexpr (FORM == FORM_DELTA) {
     B = dbase<MODEL>(psi0, p1, p2);
-    if (P.sink && smax > T(0)) sk0 = feddes(psi0, P, sa0, sda0);
+    if (has_sink) sk0 = feddes(psi0, P, sa0, sda0);
   }
   // one safeguarded step; returns true when the solve is done.  *bis: the
   // step was a bisection
@@ -640,7 +731,7 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
       float Dth, dth;
       dincr<MODEL>(B, x, p1, p2, P, Dth, dth);
       T DS = T(0), dS = T(0);
-      if (P.sink && smax > T(0)) {
+      if (has_sink) {
         T a1, da1;
         const int k1 = feddes(psi0 + x, P, a1, da1);
         DS = (k1 == sk0) ? smax * da1 * x : smax * (a1 - sa0);
@@ -651,7 +742,8 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
     } else {
       T th, dth, S, dS;
       law.eval(x, P, th, dth);
-      sink_direct(x, smax, P, S, dS);
+      S = dS = T(0);
+      if (SINK != 0) sink_direct(x, smax, P, S, dS);
       val = P.a * th + S;
       der = P.a * dth + dS;
     }
@@ -680,20 +772,52 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
     }
     return false;
   };
-  bool bis = false, done = false;
-#pragma unroll(NK > 0 ? NK : 1)
-  for (int it = 0; it < maxit; ++it) {
-    if (step(&bis)) { done = true; break; }
-  }
-  if constexpr (FORM == FORM_DELTA) {
-    if (P.newton_k > 0 && !done)
+  bool bis = false;
+  if constexpr (NK > 0) {
+    bool done = false;
+#pragma unroll(NK)
+    for (int it = 0; it < NK; ++it) {
+      if (step(&bis)) { done = true; break; }
+    }
+    if (FORM == FORM_DELTA && !done) {
+#pragma unroll 1
       for (int e = 0; e < BISECT_EXTRA && bis; ++e)
         if (step(&bis)) break;
+    }
+  } else {
+    // one copy of the step (the cycles of small levels are bound by their
+    // warps' instruction streams)
+    int left = maxit, extra = FORM == FORM_DELTA && P.newton_k > 0 ? BISECT_EXTRA : 0;
+#pragma unroll 1
+    while (!step(&bis)) {
+      if (--left > 0) continue;
+      if (!bis || extra-- <= 0) break;
+    }
   }
   return x;
 }
 
-template <typename T, int FORM, int MODEL, int NK = 0>
+// the point solve of a cell of material m: FP64 layered soils run it once
+// with the lane's own law (LawCell<COMPOSITE>), FP32 ones law by law
+template <typename T, int FORM, int MODEL, int NK = 0, int SINK = -1>
+__device__ __forceinline__ T point_solve_of(const Level<T>& L, unsigned m, T cc, T f, T x0, T psi0, T p1, T p2, T smax,
+                                            const Phys<T>& P) {
+  if constexpr (FORM == FORM_DELTA) {
+    return with_law<MODEL>(P, m, [&](auto law, const Phys<T>& Q) {
+      return point_solve<T, FORM, decltype(law)::value, NK, SINK>(cc, f, x0, psi0, p1, p2, smax, Q, LawCell<-1>{});
+    });
+  } else if constexpr (MODEL == COMPOSITE) {
+    Phys<T> Q = P;
+    Q.ts = P.mats[m].ts;
+    Q.tr = P.mats[m].tr;
+    return point_solve<T, FORM, MODEL, NK, SINK>(cc, f, x0, psi0, p1, p2, smax, Q, LawCell<MODEL>(p1, p2, m, Q));
+  } else {
+    return point_solve<T, FORM, MODEL, NK, SINK>(cc, f, x0, psi0, p1, p2, smax, P,
+                                                 LawCell<MODEL>(p1, p2, !L.p1 && !L.p2, P));
+  }
+}
+
+template <typename T, int FORM, int MODEL, int NK = 0, int SINK = -1>
 __device__ __forceinline__ void point_update(const Level<T>& L, const Phys<T>& P, long long i,
                                              int i0, int i1, int i2) {
   T mii, off;
@@ -704,11 +828,9 @@ __device__ __forceinline__ void point_update(const Level<T>& L, const Phys<T>& P
   const T f = L.g[q] + off + P.kappa * ui;
   const T p1 = L.p1 ? L.p1[q] : P.p1;
   const T p2 = L.p2 ? L.p2[q] : P.p2;
-  const T smax = L.smax ? L.smax[q] : T(0);
+  const T smax = SINK != 0 && L.smax ? L.smax[q] : T(0);
   const T psi0 = FORM == FORM_DELTA ? L.psi0[q] : T(0);
-  L.u[i] = with_law<MODEL>(P, mat_of<MODEL>(L, i), [&](auto law, const Phys<T>& Q) {
-    return point_solve<T, FORM, decltype(law)::value, NK>(cc, f, ui, psi0, p1, p2, smax, Q);
-  });
+  L.u[i] = point_solve_of<T, FORM, MODEL, NK, SINK>(L, mat_of<MODEL>(L, i), cc, f, ui, psi0, p1, p2, smax, P);
 }
 
 // Operands of one point update, gathered before any of them is used, so that
@@ -792,10 +914,8 @@ __device__ __forceinline__ void cell_sums(const Level<T>& L, const CellOps<T>& c
 // g_i - N(u)_i of a gathered cell at the value x of u_i, with its sums dg, of
 // (the expression of apply_N(), so both give the same bits)
 template <typename T, int FORM, int MODEL>
-__device__ __forceinline__ T cell_defect(const Phys<T>& P, const CellOps<T>& c, T dg, T of, T x) {
-  const T val = with_law<MODEL>(P, c.mat, [&](auto law, const Phys<T>& Q) {
-    return storage<T, FORM, decltype(law)::value>(x, c.psi0, c.p1, c.p2, c.smax, Q);
-  });
+__device__ __forceinline__ T cell_defect(const Level<T>& L, const Phys<T>& P, const CellOps<T>& c, T dg, T of, T x) {
+  const T val = storage<T, FORM, MODEL>(L, x, c.psi0, c.p1, c.p2, c.smax, c.mat, P);
   return c.g - (val + P.xi * x + dg * x - of);
 }
 
@@ -803,9 +923,7 @@ template <typename T, int FORM, int MODEL, int NK = 0, bool YZI = false>
 __device__ __forceinline__ T solve_cell_sums(const Level<T>& L, const Phys<T>& P, const CellOps<T>& c, T dg, T of) {
   const T cc = P.xi + P.kappa + dg;
   const T f = c.g + of + P.kappa * c.ui;
-  return with_law<MODEL>(P, c.mat, [&](auto law, const Phys<T>& Q) {
-    return point_solve<T, FORM, decltype(law)::value, NK>(cc, f, c.ui, c.psi0, c.p1, c.p2, c.smax, Q);
-  });
+  return point_solve_of<T, FORM, MODEL, NK>(L, c.mat, cc, f, c.ui, c.psi0, c.p1, c.p2, c.smax, P);
 }
 
 template <typename T, int FORM, int MODEL, int NK = 0, bool YZI = false>
@@ -826,9 +944,7 @@ __device__ __forceinline__ T apply_N(const Level<T>& L, const Phys<T>& P, const 
   const T p2 = L.p2 ? L.p2[q] : P.p2;
   const T smax = L.smax ? L.smax[q] : T(0);
   const T psi0 = FORM == FORM_DELTA ? L.psi0[q] : T(0);
-  const T val = with_law<MODEL>(P, mat_of<MODEL>(L, i), [&](auto law, const Phys<T>& Q) {
-    return storage<T, FORM, decltype(law)::value>(u[i], psi0, p1, p2, smax, Q);
-  });
+  const T val = storage<T, FORM, MODEL>(L, u[i], psi0, p1, p2, smax, mat_of<MODEL>(L, i), P);
   return val + P.xi * u[i] + mii * u[i] - off;
 }
 

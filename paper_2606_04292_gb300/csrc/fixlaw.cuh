@@ -48,6 +48,8 @@
 #pragma once
 
 #ifdef __CUDACC__
+#include <cmath>
+
 #include "fp64math.cuh"
 #define RICH_FD __device__ __forceinline__
 #else
@@ -262,6 +264,27 @@ RICH_FD Prep prep(double p1, double p2) {
   return q;
 }
 
+// The same on the host, for parameters known before a launch (a uniform soil,
+// a material): log2 in extended precision, the reciprocal by exact division.
+#ifdef __CUDACC__
+inline Prep host_prep(bool vg, double p1, double p2) {
+  Prep q{0, 0, 0, false};
+  const double ap = std::fabs(p1);
+  if (!(p1 > 0.0) || !(ap > 0x1p-100 && ap < 0x1p100)) return q;
+  if (!(p2 >= 1.0 / 32 && p2 < 16.0) || (vg && !(p2 > 1.0))) return q;
+  q.la = (i64)std::llrintl(std::log2((long double)p1) * 0x1p56L);
+  q.N = (u64)(p2 * 0x1p58);            // exact: p2 has 53 bits and is at least 2^-5
+  if (vg) {
+    int e;
+    const u64 m = (u64)(std::frexp(p2, &e) * 0x1p53);               // p2 = m 2^(e - 53)
+    const unsigned __int128 inv = ((unsigned __int128)1 << 117) / m;   // 2^64 / p2 = 2^(117 - e) / m
+    q.M = 0ull - (u64)(inv >> e);
+  }
+  q.ok = true;
+  return q;
+}
+#endif
+
 // theta's exponent: Se = 2^-u (scale 2^56)
 template <bool VG>
 RICH_FD u64 se_exponent(const Pow& p, u64 M) {
@@ -280,6 +303,14 @@ RICH_FD void se_slope(const Prep& q, u64 hb, bool& ok, double& Se, double& s) {
   const u64 w = shr(p.l1, 5 + p.s) + (u64)(t < 0 ? -t : 0);
   const i64 D = (i64)(w >> 2) + (i64)(u >> 2) + (lh >> 2);
   s = to_double_1(exp2_neg((int)(D >> 54), (u64)D << 10));
+}
+
+// Se alone of a prepared law
+template <bool VG>
+RICH_FD double se_prepared(const Prep& q, u64 hb, bool& ok) {
+  const i64 lh = log2_fix(hb, ok);
+  const i64 t = VG ? scale_log(q.N, add_log(q.la, lh, ok), ok) : add_log(scale_log(q.N, lh, ok), -q.la, ok);
+  return to_double_1(exp2_neg56(se_exponent<VG>(pow_log1p(t), q.M)));
 }
 
 // Se alone, from alpha (p1), n (p2) and h
@@ -350,14 +381,41 @@ RICH_FD double kr_vangenuchten(double alpha, double n, double l, u64 hb, bool& o
   return to_double(v);
 }
 
-// e^-(alpha h)
-RICH_FD double exp_gardner(double alpha, u64 hb, bool& ok) {
+// e^-(alpha h) = 2^-u: u at scale 2^56
+RICH_FD u64 gardner_exponent(double alpha, u64 hb, bool& ok) {
   const u64 ab = dbits(alpha);
   const int e = (int)(ab >> 52) + (int)(hb >> 52) - 2046;
   ok = ok && normal_pos(ab) && normal_pos(hb) && e < 6;
   const u64 P = mh((ab << 11) | 0x8000000000000000ull, (hb << 11) | 0x8000000000000000ull);   // scale 2^62
   const u64 u = mh(P, LOG2E_63);                                   // scale 2^61
-  return to_double_1(exp2_neg56(e > 5 ? 0 : shr(u, 5 - e)));
+  return e > 5 ? 0 : shr(u, 5 - e);
+}
+RICH_FD double exp_gardner(double alpha, u64 hb, bool& ok) {
+  return to_double_1(exp2_neg56(gardner_exponent(alpha, hb, ok)));
+}
+
+// Any of the three laws, chosen by lane (layered soils): one instruction
+// stream for Haverkamp's and van Genuchten's powers (they differ in where
+// log2 alpha enters and in the factor m), and Gardner's exponent selected
+// before the common 2^-u; a warp that holds several materials then takes one
+// law's time instead of their sum.  q: prep of the material (Gardner: N = 1,
+// la = 0).  slope: also d Se/d psi without its factor.
+enum { ANY_HAVERKAMP = 0, ANY_GARDNER = 1, ANY_VANGENUCHTEN = 2 };
+template <bool SLOPE>
+RICH_FD void se_any(int law, const Prep& q, double alpha, u64 hb, bool& ok, double& Se, double& s) {
+  const i64 lh = log2_fix(hb, ok);
+  const i64 x = add_log(lh, law == ANY_VANGENUCHTEN ? q.la : 0, ok);
+  const i64 t = add_log(scale_log(q.N, x, ok), law == ANY_HAVERKAMP ? -q.la : 0, ok);
+  const Pow p = pow_log1p(t);
+  u64 u = law == ANY_VANGENUCHTEN ? mh(q.M, p.L1) : p.L1;
+  if (law == ANY_GARDNER) u = gardner_exponent(alpha, hb, ok);
+  Se = to_double_1(exp2_neg56(u));
+  if (SLOPE) {
+    const u64 w = shr(p.l1, 5 + p.s) + (u64)(t < 0 ? -t : 0);
+    const i64 D = (i64)(w >> 2) + (i64)(u >> 2) + (lh >> 2);
+    s = to_double_1(exp2_neg((int)(D >> 54), (u64)D << 10));
+    if (law == ANY_GARDNER) s = Se;
+  }
 }
 
 // ---------------------------------------------------------------------------

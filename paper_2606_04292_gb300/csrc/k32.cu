@@ -22,6 +22,10 @@ void tail32(const Level<float>* dLs, const Xfer<float>* dXs, int l0, int nl, con
             int ordering, cudaStream_t s) {
   D::tail(dLs, dXs, l0, nl, ts, P, model, nu1, nu2, cmax, crtol, gamma, gamma_levels, stats, ordering, s);
 }
+void team_setup32(const Level<float>* dLs, const Xfer<float>* dXs, int nl, int ts, int blocks, bool psi0,
+                  const double* const* kb, cudaStream_t s) {
+  D::team_setup(dLs, dXs, nl, ts, blocks, psi0, kb, s);
+}
 int coop_max_blocks32(int model) { return D::coop_max_blocks(model); }
 cudaError_t coop32(const Level<float>* dLs, const Xfer<float>* dXs, int l0, int nl, int tail_start,
                    const Phys<float>& P, int model, int nu1, int nu2, int cmax, float crtol, int gamma,

@@ -26,6 +26,9 @@ void tail64(const Level<double>* dLs, const Xfer<double>* dXs, int l0, int nl, c
             int ordering, cudaStream_t s) {
   D::tail(dLs, dXs, l0, nl, ts, P, model, nu1, nu2, cmax, crtol, gamma, gamma_levels, stats, ordering, s);
 }
+void team_setup64(const Level<double>* dLs, const Xfer<double>* dXs, int nl, int ts, int blocks, cudaStream_t s) {
+  D::team_setup(dLs, dXs, nl, ts, blocks, false, nullptr, s);
+}
 void sweep_lex64(const Level<double>& L, const Phys<double>& P, int model, cudaStream_t s) { D::sweep_lex(L, P, model, s); }
 
 // ---------------------------------------------------------------------------
@@ -47,42 +50,44 @@ __global__ void __launch_bounds__(256) k_prep_lagged(long long n, const double* 
   // evaluations (nullable: evaluate here, and keep them in *_out if given).
   // Kcf (nullable): an FP32 copy of Kc for the inner cycles of the mixed
   // mode; predict: the iterate starts at psi* instead of psi^n.
+  const bool uniform = !p1f && !p2f;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double p1 = p1f ? p1f[i] : P.p1, p2 = p2f ? p2f[i] : P.p2;
     const double ks = Ks ? Ks[i] : Ks_s;
     const double pn = psin[i];
-    with_law<MODEL>(P, mat_at<MODEL>(mat, i), [&](auto law, const Phys<double>& Q) {
-      constexpr int ML = decltype(law)::value;
-      double thn;
-      if (thn_in) {
-        thn = thn_in[i];
+    const unsigned mi = mat_at<MODEL>(mat, i);
+    // (theta_cell, as in the defect kernel, so that a cache filled here and
+    // one filled there hold the same bits for the same state)
+    double thn;
+    if (thn_in) {
+      thn = thn_in[i];
+    } else {
+      thn = theta_cell<MODEL>(pn, p1, p2, mi, uniform, P);
+      if (thn_out) thn_out[i] = thn;
+    }
+    double ps, hist;
+    if (scheme == 1) {
+      ps = pn;
+      hist = thn * hist_scale;
+    } else {
+      const double pm = psinm1[i];
+      double thm;
+      if (thm_in) {
+        thm = thm_in[i];
       } else {
-        thn = theta_only_d<ML>(pn, p1, p2, Q);
-        if (thn_out) thn_out[i] = thn;
+        thm = theta_cell<MODEL>(pm, p1, p2, mi, uniform, P);
+        if (thm_out) thm_out[i] = thm;
       }
-      double ps, hist;
-      if (scheme == 1) {
-        ps = pn;
-        hist = thn * hist_scale;
-      } else {
-        const double pm = psinm1[i];
-        double thm;
-        if (thm_in) {
-          thm = thm_in[i];
-        } else {
-          thm = theta_only_d<ML>(pm, p1, p2, Q);
-          if (thm_out) thm_out[i] = thm;
-        }
-        ps = P.lag ? pn : 2.0 * pn - pm;
-        hist = (4.0 * thn - thm) * hist_scale;
-      }
-      const double K = cond_d<ML>(ps, p1, p2, ks, Q);
-      Kc[i] = K;
-      if (Kcf) Kcf[i] = (float)K;
-      g[i] = hist + P.xi * ps;
-      u[i] = predict ? ps : pn;
-      return 0;
+      ps = P.lag ? pn : 2.0 * pn - pm;
+      hist = (4.0 * thn - thm) * hist_scale;
+    }
+    const double K = with_law<MODEL>(P, mi, [&](auto law, const Phys<double>& Q) {
+      return cond_d<decltype(law)::value>(ps, p1, p2, ks, Q);
     });
+    Kc[i] = K;
+    if (Kcf) Kcf[i] = (float)K;
+    g[i] = hist + P.xi * ps;
+    u[i] = predict ? ps : pn;
   }
 }
 
@@ -257,26 +262,6 @@ __global__ void __launch_bounds__(256) k_prep_rhs_dd(Geom G, BcDev bc, const dou
   }
 }
 
-// restriction of a boundary-face array over the face's two in-plane axes
-template <typename T>
-__global__ void __launch_bounds__(256) k_restrict_face(Geom F, Geom C, Xfer<T> X, int ax, const T* fine, T* coarse) {
-  int oa[2], k = 0;
-  for (int a = 0; a < 3; ++a)
-    if (a != ax) oa[k++] = a;
-  const int nF[3] = {F.n0, F.n1, F.n2}, nC[3] = {C.n0, C.n1, C.n2};
-  const long long nc = (long long)nC[oa[0]] * nC[oa[1]];
-  for (long long J = blockIdx.x * (long long)blockDim.x + threadIdx.x; J < nc; J += (long long)gridDim.x * blockDim.x) {
-    const int J0 = (int)(J % nC[oa[0]]), J1 = (int)(J / nC[oa[0]]);
-    const int c0 = X.rc[oa[0]][J0], c1 = X.rc[oa[1]][J1];
-    T s = T(0);
-    for (int a1 = 0; a1 < c1; ++a1)
-      for (int a0 = 0; a0 < c0; ++a0)
-        s += X.rw[oa[0]][RMAX * J0 + a0] * X.rw[oa[1]][RMAX * J1 + a1] *
-             fine[X.ri[oa[0]][RMAX * J0 + a0] + (long long)nF[oa[0]] * X.ri[oa[1]][RMAX * J1 + a1]];
-    coarse[J] = s;
-  }
-}
-
 // Sink coefficient (reading): Tp exp(-depth/decay) normalised over the root
 // zone [0, root_depth], depth measured down from the top face.
 __global__ void __launch_bounds__(256) k_sink_coef(Geom G, double Tp, double D, double lam, double* smax) {
@@ -416,9 +401,7 @@ __global__ void __launch_bounds__(256) k_outer_residual64(Level<double> L, Phys<
       th = th_in[i];
     } else {
       const double p1 = L.p1 ? L.p1[i] : P.p1, p2 = L.p2 ? L.p2[i] : P.p2;
-      th = with_law<MODEL>(P, mat_of<MODEL>(L, i), [&](auto law, const Phys<double>& Q) {
-        return theta_only_d<decltype(law)::value>(ui, p1, p2, Q);
-      });
+      th = theta_cell<MODEL>(ui, p1, p2, mat_of<MODEL>(L, i), !L.p1 && !L.p2, P);
       if (th_out) th_out[i] = th;
     }
     double S, dS;
@@ -498,24 +481,6 @@ void prep_rhs_dd(const Geom& G, const BcDev& bc, const double* Ks, double Ks_s, 
     k_prep_rhs_dd<decltype(m)::value><<<b, 256, 0, s>>>(G, bc, Ks, ks, p1, p2, mat, P, Q, H, Kc, g, kb[0], kb[1], kb[2],
                                                         kb[3], kb[4], kb[5]);
   });
-}
-
-void restrict_face64(const Geom& F, const Geom& C, const Xfer<double>& X, int axis, const double* fine,
-                     double* coarse, cudaStream_t s) {
-  const int nC[3] = {C.n0, C.n1, C.n2};
-  long long nc = 1;
-  for (int a = 0; a < 3; ++a)
-    if (a != axis) nc *= nC[a];
-  k_restrict_face<double><<<grid_for(nc), 256, 0, s>>>(F, C, X, axis, fine, coarse);
-}
-
-void restrict_face32(const Geom& F, const Geom& C, const Xfer<float>& X, int axis, const float* fine, float* coarse,
-                     cudaStream_t s) {
-  const int nC[3] = {C.n0, C.n1, C.n2};
-  long long nc = 1;
-  for (int a = 0; a < 3; ++a)
-    if (a != axis) nc *= nC[a];
-  k_restrict_face<float><<<grid_for(nc), 256, 0, s>>>(F, C, X, axis, fine, coarse);
 }
 
 void sink_coef(const Geom& G, double Tp, double depth, double decay, double* smax, cudaStream_t s) {
@@ -753,22 +718,19 @@ __global__ void __launch_bounds__(256) k_mass_balance64(Level<double> L, Geom G,
     const double p1 = L.p1 ? L.p1[i] : P.p1, p2 = L.p2 ? L.p2[i] : P.p2;
     const double psi = L.u[i], pn = psin[i];
     const unsigned mi = mat_of<MODEL>(L, i);
-    double th1, hist, ps;
-    with_law<MODEL>(P, mi, [&](auto law, const Phys<double>& Q) {
-      constexpr int ML = decltype(law)::value;
-      th1 = th_new ? th_new[i] : theta_only_d<ML>(psi, p1, p2, Q);
-      const double thn = th_n ? th_n[i] : theta_only_d<ML>(pn, p1, p2, Q);
-      if (scheme == 1) {
-        hist = thn * hist_scale;
-        ps = pn;
-      } else {
-        const double pm = psinm1[i];
-        const double thm = th_nm1 ? th_nm1[i] : theta_only_d<ML>(pm, p1, p2, Q);
-        hist = (4.0 * thn - thm) * hist_scale;
-        ps = Q.lag ? pn : 2.0 * pn - pm;
-      }
-      return 0;
-    });
+    const bool uniform = !L.p1 && !L.p2;
+    const double th1 = th_new ? th_new[i] : theta_cell<MODEL>(psi, p1, p2, mi, uniform, P);
+    const double thn = th_n ? th_n[i] : theta_cell<MODEL>(pn, p1, p2, mi, uniform, P);
+    double hist, ps;
+    if (scheme == 1) {
+      hist = thn * hist_scale;
+      ps = pn;
+    } else {
+      const double pm = psinm1[i];
+      const double thm = th_nm1 ? th_nm1[i] : theta_cell<MODEL>(pm, p1, p2, mi, uniform, P);
+      hist = (4.0 * thn - thm) * hist_scale;
+      ps = P.lag ? pn : 2.0 * pn - pm;
+    }
     const double smax = L.smax ? L.smax[i] : 0.0;
     double S, dS;
     sink_direct(psi, smax, P, S, dS);

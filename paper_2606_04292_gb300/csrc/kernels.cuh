@@ -77,7 +77,7 @@ __device__ __forceinline__ unsigned long long sweep_pipe_body(const Level<T>& L,
       const T x = solve_cell_sums<T, FORM, MODEL, NK, YZI>(L, P, cur, dg, of);
       L.u[cur.i] = x;
       if (RESID) {
-        const T di = cell_defect<T, FORM, MODEL>(P, cur, dg, of, x);
+        const T di = cell_defect<T, FORM, MODEL>(L, P, cur, dg, of, x);
         L.d[cur.i] = di;
         const unsigned long long b = nbits(di);
         mx = b > mx ? b : mx;
@@ -516,7 +516,6 @@ struct BlockTeam {
 
 // Shared memory of a cluster team: block_max's words and two rotating rows of
 // one maximum per block.
-constexpr int CLUSTER_MAX = 16;
 struct ClusterShared {
   unsigned long long sm[33];
   unsigned long long part[2][CLUSTER_MAX];
@@ -602,7 +601,9 @@ struct GridTeam {
 
 // one NGS sweep of a level by a team: red then black half-sweeps (ordering
 // 1), or the lexicographic order hyperplane by hyperplane (0).  One copy of
-// the point update serves both.
+// the point update serves both; the update without a sink is its own (the
+// sink's pieces, if-converted, cost the 128-cell column 5%), but in the
+// columns, whose second copy would spill (48.1 -> 50.2 ms).
 template <typename T, int FORM, int MODEL, typename TM>
 __device__ __forceinline__ void team_sweep(const Level<T>& L, const Phys<T>& P, int ordering, TM& tm) {
   const unsigned rows = (unsigned)L.n1 * (unsigned)L.n2;
@@ -622,7 +623,14 @@ __device__ __forceinline__ void team_sweep(const Level<T>& L, const Phys<T>& P, 
         on = i0 >= 0 && i0 < L.n0;
         i = (unsigned)i0 + (unsigned)L.n0 * t;
       }
-      if (on) point_update<T, FORM, MODEL>(L, P, i, i0, i1, i2);
+      if (on) {
+        if constexpr (TM::splits) {
+          if (L.smax) point_update<T, FORM, MODEL, 0, 1>(L, P, i, i0, i1, i2);
+          else point_update<T, FORM, MODEL, 0, 0>(L, P, i, i0, i1, i2);
+        } else {
+          point_update<T, FORM, MODEL>(L, P, i, i0, i1, i2);
+        }
+      }
     }
     tm.sync();
   }
@@ -813,6 +821,78 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail(const Level<T>* __rest
                              gamma_levels, updates, ordering, handoff, tm);
   if (threadIdx.x == 0 && tm.lead() && stats) atomicAdd(stats, updates);
   tm.sync();                           // (no block leaves while another may still write to its shared memory)
+}
+
+// One coarse cell of a boundary-face array of axis ax: the restriction over the
+// face's two in-plane axes.
+template <typename T>
+__device__ __forceinline__ T restrict_face_at(const int* nF, const int* nC, const Xfer<T>& X, int ax,
+                                              const T* __restrict__ fine, int J) {
+  const int o0 = ax == 0 ? 1 : 0, o1 = ax == 2 ? 1 : 2;
+  const int J1 = J / nC[o0], J0 = J - J1 * nC[o0];
+  const int c0 = X.rc[o0][J0], c1 = X.rc[o1][J1];
+  T s = T(0);
+  for (int a1 = 0; a1 < c1; ++a1)
+    for (int a0 = 0; a0 < c0; ++a0)
+      s += X.rw[o0][RMAX * J0 + a0] * X.rw[o1][RMAX * J1 + a1] *
+           fine[X.ri[o0][RMAX * J0 + a0] + (long long)nF[o0] * X.ri[o1][RMAX * J1 + a1]];
+  return s;
+}
+
+// FP64 boundary conductances of the finest level whose FP32 copies the FP32
+// set-up makes first (null: FP64 levels, or none)
+struct FaceSource {
+  const double* kb[6];
+};
+
+// The per-step set-up of the coarse levels in one cluster: every level's
+// boundary conductances and, from level ts on, the lagged conductivity
+// (psi0 false), or the frozen state (psi0 true) of the levels from ts on.  One
+// launch instead of up to seven per level, each of which takes a launch's ~2
+// us whatever its size; the values of the launches it replaces.
+template <typename T>
+__global__ void __launch_bounds__(TAIL_THREADS, 1) k_team_setup(const Level<T>* __restrict__ Ls,
+                                                                const Xfer<T>* __restrict__ Xs, int nl, int ts,
+                                                                bool psi0, FaceSource src) {
+  __shared__ ClusterShared sh;
+  __shared__ Level<T> sL[TEAM_LEVELS];
+  __shared__ Xfer<T> sX[TEAM_LEVELS];
+  stage_levels(Ls, Xs, 0, nl, sL, sX);
+  ClusterTeam tm(&sh);
+  tm.sync();
+  const int nface = 2 * sL[0].dim;
+  if (!psi0 && src.kb[0]) {
+    for (int f = 0; f < nface; ++f) {
+      const int n[3] = {sL[0].n0, sL[0].n1, sL[0].n2};
+      const unsigned cells = (unsigned)(sL[0].ncell / n[f >> 1]);
+      for (unsigned i = tm.rank(); i < cells; i += tm.size()) const_cast<T*>(sL[0].kb[f])[i] = (T)src.kb[f][i];
+    }
+    tm.sync();
+  }
+  const GridLevels<T> lv{sL, sX, 0, nl};
+  for (int l = psi0 ? ts : 0; l + 1 < nl; ++l) {
+    const Level<T>& F = sL[l];
+    const Level<T>& C = sL[l + 1];
+    if (!psi0) {
+      const int nF[3] = {F.n0, F.n1, F.n2}, nC[3] = {C.n0, C.n1, C.n2};
+      for (int f = 0; f < nface; ++f) {
+        const unsigned cells = (unsigned)(C.ncell / nC[f >> 1]);
+        for (unsigned J = tm.rank(); J < cells; J += tm.size())
+          const_cast<T*>(C.kb[f])[J] = restrict_face_at(nF, nC, sX[l], f >> 1, F.kb[f], (int)J);
+      }
+    }
+    if (l >= ts) {
+      const T* from = psi0 ? F.psi0 : F.Kc;
+      T* to = const_cast<T*>(psi0 ? C.psi0 : C.Kc);
+      for (unsigned J = tm.rank(); J < (unsigned)C.ncell; J += tm.size()) {
+        int J0, J1, J2;
+        cell_coords(C, J, J0, J1, J2);
+        to[J] = lv.nested(l) ? restrict_nested_at(F, C, from, J0, J1, J2) : restrict_at(F, sX[l], from, J0, J1, J2);
+      }
+    }
+    tm.sync();
+  }
+  tm.sync();
 }
 
 // The coarse levels of a big grid as one cooperative launch, a grid barrier
@@ -1017,6 +1097,12 @@ struct Dispatch {
       k_prolong_nested<T><<<g.grid, g.block, 0, s>>>(F, C, X);
     else
       k_prolong<T><<<g.grid, g.block, 0, s>>>(F, C, X);
+  }
+  static void team_setup(const Level<T>* dLs, const Xfer<T>* dXs, int nl, int ts, int blocks, bool psi0,
+                         const double* const* kb, cudaStream_t s) {
+    FaceSource src{};
+    for (int f = 0; kb && f < 6; ++f) src.kb[f] = kb[f];
+    launch_cluster(k_team_setup<T>, blocks, 1, TAIL_THREADS, s, dLs, dXs, nl, ts, psi0, src);
   }
   // the cooperative coarse cycle: the most blocks that can be co-resident
   static int coop_max_blocks(int model) {

@@ -28,6 +28,7 @@ struct Geom {
 // How the coarse tail runs: one cluster of `blocks` blocks; levels from
 // `handoff` on by its first block alone; transfers below `tail_start` as the
 // grid kernels take them (nested formulas), from it on through the tables.
+constexpr int CLUSTER_MAX = 16;
 struct TeamShape {
   int blocks, handoff, tail_start;
 };
@@ -43,7 +44,7 @@ inline TeamShape team_shape(const long long* cells, int l0, int nl, int tail_sta
   const long long solo = sizeof(T) == 8 ? 256 : 1024, per = sizeof(T) == 8 ? 128 : 256;
   TeamShape ts{1, l0, tail_start};
   if (cells[l0] <= solo) return ts;
-  while (ts.blocks < 16 && ts.blocks * per < cells[l0]) ts.blocks *= 2;
+  while (ts.blocks < CLUSTER_MAX && ts.blocks * per < cells[l0]) ts.blocks *= 2;
   ts.handoff = nl;
   for (int l = l0; l < nl; ++l)
     if (cells[l] <= solo) { ts.handoff = l; break; }
@@ -92,6 +93,13 @@ void prolong32(const Level<float>& F, const Level<float>& C, const Xfer<float>& 
 void tail32(const Level<float>* dLs, const Xfer<float>* dXs, int l0, int nl, const TeamShape& ts,
             const Phys<float>& P, int model, int nu1, int nu2, int cmax, float crtol, int gamma, int gamma_levels,
             unsigned long long* stats, int ordering, cudaStream_t s);
+// the coarse levels' share of the per-step set-up in one cluster of `blocks`
+// blocks (k_team_setup): boundary conductances of every level and Kc from
+// level ts on, or psi0 from level ts on; kb: the finest level's FP64 boundary
+// conductances, converted first (FP32 levels; null otherwise)
+void team_setup32(const Level<float>* dLs, const Xfer<float>* dXs, int nl, int ts, int blocks, bool psi0,
+                  const double* const* kb, cudaStream_t s);
+void team_setup64(const Level<double>* dLs, const Xfer<double>* dXs, int nl, int ts, int blocks, cudaStream_t s);
 void sweep_lex32(const Level<float>& L, const Phys<float>& P, int model, cudaStream_t s);
 // the cycle from level l0 down as one cooperative launch of `blocks` blocks
 // (levels from tail_start on take the single-block tail's transfers); slots:
@@ -123,8 +131,6 @@ void prep_rhs(const Geom& G, const BcDev& bc, const double* Ks, double Ks_s, con
 void prep_rhs_dd(const Geom& G, const BcDev& bc, const double* Ks, double Ks_s, const double* p1, const double* p2,
                  const uint8_t* mat, const Phys<double>& P, const DDPhys& Q, int model, const double* Kc, double* g,
                  double* const kb[6], cudaStream_t s);
-void restrict_face64(const Geom& F, const Geom& C, const Xfer<double>& X, int axis, const double* fine,
-                     double* coarse, cudaStream_t s);
 void sink_coef(const Geom& G, double Tp, double depth, double decay, double* smax, cudaStream_t s);
 void to_float(const double* src, float* dst, long long n, cudaStream_t s);
 
@@ -158,8 +164,6 @@ int mass_balance(const Level<double>& L, const Geom& G, const BcDev& bc, const P
                  int model, const double* psin, const double* psinm1, int scheme, double dt, const double* th_new,
                  const double* th_n, const double* th_nm1, double* part, unsigned* dmin_bits, bool fp64,
                  cudaStream_t s);
-void restrict_face32(const Geom& F, const Geom& C, const Xfer<float>& X, int axis, const float* fine, float* coarse,
-                     cudaStream_t s);
 void apply_delta(double* u, const float* delta, long long n, cudaStream_t s);
 // y = f(x) elementwise for the laws' FP64 elementary functions (fn 0..3:
 // exp, expm1, log, log1p) or CUDA's (fn 4..7), device arrays

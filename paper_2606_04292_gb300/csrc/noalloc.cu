@@ -121,9 +121,8 @@ __device__ void na_prepare(const NaPlan& p, ClusterTeam& tm) {
     }
     const double pn = p.psin[i];
     const unsigned mi = mat_at<MODEL>(L.mat, i);
-    const double thn = with_law<MODEL>(P, mi, [&](auto law, const Phys<double>& Q) {
-      return theta_only_d<decltype(law)::value>(pn, p1, p2, Q);
-    });
+    const bool uniform = !p.p1_field && !p.p2_field;
+    const double thn = theta_cell<MODEL>(pn, p1, p2, mi, uniform, P);
     double ps, hist;
     if (p.scheme == 1) {
       ps = pn;
@@ -131,9 +130,7 @@ __device__ void na_prepare(const NaPlan& p, ClusterTeam& tm) {
     } else {
       const double pm = p.psinm1[i];
       ps = P.lag ? pn : 2.0 * pn - pm;
-      const double thm = with_law<MODEL>(P, mi, [&](auto law, const Phys<double>& Q) {
-        return theta_only_d<decltype(law)::value>(pm, p1, p2, Q);
-      });
+      const double thm = theta_cell<MODEL>(pm, p1, p2, mi, uniform, P);
       hist = (4.0 * thn - thm) / (2.0 * p.dt);
     }
     const double ks = p.Ks_field ? p.Ks_field[i] : p.Ks;
@@ -407,6 +404,8 @@ long long build_plan(const richards_grid* grid, const richards_soil* soil, const
   P.tr = soil->theta_r;
   P.p1 = soil->p1; P.p2 = soil->p2; P.p3 = soil->p3; P.p4 = soil->p4;
   P.h1 = sink->h1; P.h2 = sink->h2; P.h3 = sink->h3; P.h4 = sink->h4;
+  set_sink_slopes(P);
+  if (!cx || !cx->mats) P.q = law_prep(soil->model, soil->p1, soil->p2);
   P.newton_k = o.newton_iters;
   P.sink = sink->enabled;
   P.lag = o.bdf2_lag;
