@@ -22,7 +22,6 @@ namespace rich {
 namespace {
 
 constexpr int COL_MAXLEV = 14;
-constexpr int COL_THREADS_MAX = 512;
 constexpr int COL_ARRAYS = 7;      // u, ubar, g, d, Kc, psi0, smax per level (FP32)
 
 struct ColDesc {
@@ -440,8 +439,15 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
   __syncthreads();
 }
 
+// A column's phases are bound by the latency of its point updates (issue slots
+// 20% busy), so what counts is how many columns an SM holds: 80 registers a
+// thread admit three 256-thread blocks, as many as the shared memory of
+// 1024-cell columns, where 128 admitted two.  The inner solve spills 32 bytes,
+// the outer layer ~540 (once per correction).  4096 columns x 4 steps: 128
+// registers 46.7 ms, 96 47.9 (two blocks still), 80 40.0, 64 39.6; a fourth
+// length class (513-768 cells) 39.4, not taken.
 template <int MODEL>
-__global__ void __launch_bounds__(COL_THREADS_MAX, 1) k_columns(ColArgs A) {
+__global__ void __maxnreg__(80) k_columns(ColArgs A) {
   extern __shared__ float smem[];
   __shared__ Level<float> Ls[COL_MAXLEV];
   __shared__ unsigned long long sm[33];
