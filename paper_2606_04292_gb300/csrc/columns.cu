@@ -269,7 +269,7 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
       if (th_valid) {
         th = dd_split(thn[i]);
       } else {
-        th = theta_x<MODEL>(pn, Q.p1, Q.p2, Q, P64);
+        th = theta_x<MODEL>(pnd, D.p1, D.p2, 0, false, Q, P64);
         thn[i] = dd_join(th);
       }
       dd ps, hist;
@@ -279,7 +279,7 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
       } else {
         const dd pm = dd_split(psinm1[i]);
         ps = A.lag ? pn : dd_sub(mk(2.0f * pn.hi, 2.0f * pn.lo), pm);
-        hist = dd_mul(dd_sub(mk(4.0f * th.hi, 4.0f * th.lo), theta_x<MODEL>(pm, Q.p1, Q.p2, Q, P64)), hist_scale);
+        hist = dd_mul(dd_sub(mk(4.0f * th.hi, 4.0f * th.lo), theta_x<MODEL>(psinm1[i], D.p1, D.p2, 0, false, Q, P64)), hist_scale);
       }
       A.Kc[off + i] = dd_join(cond_x<MODEL>(ps, Q.p1, Q.p2, Ks, Q, P64));
       G.g[i] = dd_join(dd_add(hist, dd_mul(Q.xi, ps)));
@@ -377,7 +377,7 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
         if (outer == 0) {
           th = dd_split(thn[i]);
         } else {
-          th = theta_x<MODEL>(ui, Q.p1, Q.p2, Q, P64);
+          th = theta_x<MODEL>(G.u[i], D.p1, D.p2, 0, false, Q, P64);
           if (!A.fp64) thcur[i] = dd_join(th);     // (FP64 outer: from the FP64 defect)
         }
         const dd S = G.smax ? sink_x(ui, dd_split(G.smax[i]), Q) : mk(0.0f);
@@ -440,14 +440,15 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
 }
 
 // A column's phases are bound by the latency of its point updates (issue slots
-// 20% busy), so what counts is how many columns an SM holds: 80 registers a
+// 20% busy), so what counts is how many columns an SM holds: 72 registers a
 // thread admit three 256-thread blocks, as many as the shared memory of
-// 1024-cell columns, where 128 admitted two.  The inner solve spills 32 bytes,
+// 1024-cell columns, where 128 admitted two.  The inner solve spills 64 bytes,
 // the outer layer ~540 (once per correction).  4096 columns x 4 steps: 128
-// registers 46.7 ms, 96 47.9 (two blocks still), 80 40.0, 64 39.6; a fourth
-// length class (513-768 cells) 39.4, not taken.
+// registers 46.7 ms, 96 47.9 (two blocks still), 80 40.0, 64 39.6; with the
+// fixed-point theta 80 38.9, 72 38.0, 64 and a fourth length class (513-768
+// cells) 37.9.
 template <int MODEL>
-__global__ void __maxnreg__(80) k_columns(ColArgs A) {
+__global__ void __maxnreg__(72) k_columns(ColArgs A) {
   extern __shared__ float smem[];
   __shared__ Level<float> Ls[COL_MAXLEV];
   __shared__ unsigned long long sm[33];

@@ -307,15 +307,19 @@ RICH_FD void se_slope(const Prep& q, u64 hb, bool& ok, double& Se, double& s) {
 
 // Se alone of a prepared law
 template <bool VG>
-RICH_FD double se_prepared(const Prep& q, u64 hb, bool& ok) {
+RICH_FD u64 prepared_u(const Prep& q, u64 hb, bool& ok) {
   const i64 lh = log2_fix(hb, ok);
   const i64 t = VG ? scale_log(q.N, add_log(q.la, lh, ok), ok) : add_log(scale_log(q.N, lh, ok), -q.la, ok);
-  return to_double_1(exp2_neg56(se_exponent<VG>(pow_log1p(t), q.M)));
+  return se_exponent<VG>(pow_log1p(t), q.M);
+}
+template <bool VG>
+RICH_FD double se_prepared(const Prep& q, u64 hb, bool& ok) {
+  return to_double_1(exp2_neg56(prepared_u<VG>(q, hb, ok)));
 }
 
-// Se alone, from alpha (p1), n (p2) and h
+// Se alone, from alpha (p1), n (p2) and h: its exponent, Se = 2^-u (scale 2^56)
 template <bool VG>
-RICH_FD double se_only(double p1, double p2, u64 hb, bool& ok) {
+RICH_FD u64 se_u(double p1, double p2, u64 hb, bool& ok) {
   const u64 nb = dbits(p2);
   const u64 N = to_fix58(nb, ok);
   i64 t;
@@ -327,7 +331,11 @@ RICH_FD double se_only(double p1, double p2, u64 hb, bool& ok) {
   } else {
     t = add_log(scale_log(N, log2_fix(hb, ok), ok), -log2_fix(dbits(p1), ok), ok);
   }
-  return to_double_1(exp2_neg56(se_exponent<VG>(pow_log1p(t), M)));
+  return se_exponent<VG>(pow_log1p(t), M);
+}
+template <bool VG>
+RICH_FD double se_only(double p1, double p2, u64 hb, bool& ok) {
+  return to_double_1(exp2_neg56(se_u<VG>(p1, p2, hb, ok)));
 }
 
 // K/Ks of Haverkamp: A/(A + h^gamma)
@@ -401,14 +409,18 @@ RICH_FD double exp_gardner(double alpha, u64 hb, bool& ok) {
 // law's time instead of their sum.  q: prep of the material (Gardner: N = 1,
 // la = 0).  slope: also d Se/d psi without its factor.
 enum { ANY_HAVERKAMP = 0, ANY_GARDNER = 1, ANY_VANGENUCHTEN = 2 };
+RICH_FD u64 any_u(int law, const Prep& q, double alpha, u64 hb, bool& ok, i64& lh, i64& t, Pow& p) {
+  lh = log2_fix(hb, ok);
+  const i64 x = add_log(lh, law == ANY_VANGENUCHTEN ? q.la : 0, ok);
+  t = add_log(scale_log(q.N, x, ok), law == ANY_HAVERKAMP ? -q.la : 0, ok);
+  p = pow_log1p(t);
+  return law == ANY_GARDNER ? gardner_exponent(alpha, hb, ok) : law == ANY_VANGENUCHTEN ? mh(q.M, p.L1) : p.L1;
+}
 template <bool SLOPE>
 RICH_FD void se_any(int law, const Prep& q, double alpha, u64 hb, bool& ok, double& Se, double& s) {
-  const i64 lh = log2_fix(hb, ok);
-  const i64 x = add_log(lh, law == ANY_VANGENUCHTEN ? q.la : 0, ok);
-  const i64 t = add_log(scale_log(q.N, x, ok), law == ANY_HAVERKAMP ? -q.la : 0, ok);
-  const Pow p = pow_log1p(t);
-  u64 u = law == ANY_VANGENUCHTEN ? mh(q.M, p.L1) : p.L1;
-  if (law == ANY_GARDNER) u = gardner_exponent(alpha, hb, ok);
+  i64 lh, t;
+  Pow p;
+  const u64 u = any_u(law, q, alpha, hb, ok, lh, t, p);
   Se = to_double_1(exp2_neg56(u));
   if (SLOPE) {
     const u64 w = shr(p.l1, 5 + p.s) + (u64)(t < 0 ? -t : 0);

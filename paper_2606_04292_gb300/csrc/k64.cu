@@ -106,34 +106,37 @@ __global__ void __launch_bounds__(256) k_prep_lagged_dd(long long n, const doubl
                                                         double* thn_out, double* thm_out, bool predict) {
   // hist_scale: 1/tau (BDF1) or 1/(2 tau) (BDF2)
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const dd p1 = p1f ? dd_split(p1f[i]) : Q.p1, p2 = p2f ? dd_split(p2f[i]) : Q.p2;
+    const double p1d = p1f ? p1f[i] : P.p1, p2d = p2f ? p2f[i] : P.p2;
+    const bool uniform = !p1f && !p2f;
     const double pnd = psin[i];
     const dd pn = dd_split(pnd);
-    with_law_dd<MODEL>(P, Q, mat_at<MODEL>(mat, i), [&](auto law, const Phys<double>& Pc, const DDPhys& Qc) {
+    const unsigned mi = mat_at<MODEL>(mat, i);
+    dd thn;
+    if (thn_in) {
+      thn = dd_split(thn_in[i]);
+    } else {
+      thn = theta_x<MODEL>(pnd, p1d, p2d, mi, uniform, Q, P);
+      if (thn_out) thn_out[i] = dd_join(thn);
+    }
+    dd ps, hist;
+    if (scheme == 1) {
+      ps = pn;
+      hist = dd_mul(thn, hist_scale);
+    } else {
+      const dd pm = dd_split(psinm1[i]);
+      dd thm;
+      if (thm_in) {
+        thm = dd_split(thm_in[i]);
+      } else {
+        thm = theta_x<MODEL>(psinm1[i], p1d, p2d, mi, uniform, Q, P);
+        if (thm_out) thm_out[i] = dd_join(thm);
+      }
+      ps = P.lag ? pn : dd_sub(mk(2.0f * pn.hi, 2.0f * pn.lo), pm);
+      hist = dd_mul(dd_sub(mk(4.0f * thn.hi, 4.0f * thn.lo), thm), hist_scale);
+    }
+    const dd p1 = p1f ? dd_split(p1d) : Q.p1, p2 = p2f ? dd_split(p2d) : Q.p2;
+    with_law_dd<MODEL>(P, Q, mi, [&](auto law, const Phys<double>& Pc, const DDPhys& Qc) {
       constexpr int ML = decltype(law)::value;
-      dd thn;
-      if (thn_in) {
-        thn = dd_split(thn_in[i]);
-      } else {
-        thn = theta_x<ML>(pn, p1, p2, Qc, Pc);
-        if (thn_out) thn_out[i] = dd_join(thn);
-      }
-      dd ps, hist;
-      if (scheme == 1) {
-        ps = pn;
-        hist = dd_mul(thn, hist_scale);
-      } else {
-        const dd pm = dd_split(psinm1[i]);
-        dd thm;
-        if (thm_in) {
-          thm = dd_split(thm_in[i]);
-        } else {
-          thm = theta_x<ML>(pm, p1, p2, Qc, Pc);
-          if (thm_out) thm_out[i] = dd_join(thm);
-        }
-        ps = Pc.lag ? pn : dd_sub(mk(2.0f * pn.hi, 2.0f * pn.lo), pm);
-        hist = dd_mul(dd_sub(mk(4.0f * thn.hi, 4.0f * thn.lo), thm), hist_scale);
-      }
       const dd K = cond_x<ML>(ps, p1, p2, Ks ? dd_split(Ks[i]) : Ks_s, Qc, Pc);
       Kc[i] = dd_join(K);
       Kcf[i] = dd_float(K);
@@ -318,27 +321,31 @@ __global__ void __launch_bounds__(128) k_outer_residual_dd(Level<double> L, Phys
       if (a == 0) fc = i1 + (long long)L.n1 * i2;
       else if (a == 1) fc = i0 + (long long)L.n0 * i2;
       else fc = i0 + (long long)L.n0 * i1;
-      if (ii[a] > 0) {
+      // (both faces' (K_i + K_j)(u_i - u_j), then one factor 1/(2 h^2))
+      const bool lo = ii[a] > 0, hi = ii[a] < nn[a] - 1;
+      dd q = mk(0.0f);
+      if (lo) {
         const long long j = i - st[a];
-        flux = dd_add(flux, dd_mul(dd_mul(dd_add(Ki, dd_split(K[j])), hs), dd_sub(ui, dd_split(u[j]))));
+        q = dd_mul(dd_add(Ki, dd_split(K[j])), dd_sub(ui, dd_split(u[j])));
       } else {
         db = dd_add(db, dd_mul(dd_split(L.kb[2 * a][fc]), s2));
       }
-      if (ii[a] < nn[a] - 1) {
+      if (hi) {
         const long long j = i + st[a];
-        flux = dd_add(flux, dd_mul(dd_mul(dd_add(Ki, dd_split(K[j])), hs), dd_sub(ui, dd_split(u[j]))));
+        const dd r = dd_mul(dd_add(Ki, dd_split(K[j])), dd_sub(ui, dd_split(u[j])));
+        q = lo ? dd_add(q, r) : r;
       } else {
         db = dd_add(db, dd_mul(dd_split(L.kb[2 * a + 1][fc]), s2));
       }
+      q = dd_mul(q, hs);
+      flux = a == 0 ? q : dd_add(flux, q);
     }
     dd th;
     if (th_in) {
       th = dd_split(th_in[i]);
     } else {
-      const dd p1 = L.p1 ? dd_split(L.p1[i]) : Q.p1, p2 = L.p2 ? dd_split(L.p2[i]) : Q.p2;
-      th = with_law_dd<MODEL>(P, Q, mat_of<MODEL>(L, i), [&](auto law, const Phys<double>& Pc, const DDPhys& Qc) {
-        return theta_x<decltype(law)::value>(ui, p1, p2, Qc, Pc);
-      });
+      th = theta_x<MODEL>(u[i], L.p1 ? L.p1[i] : P.p1, L.p2 ? L.p2[i] : P.p2, mat_of<MODEL>(L, i), !L.p1 && !L.p2, Q,
+                          P);
       if (th_out) th_out[i] = dd_join(th);
     }
     const dd S = L.smax ? sink_x(ui, dd_split(L.smax[i]), Q) : mk(0.0f);
@@ -548,9 +555,11 @@ __global__ void __launch_bounds__(256) k_soil_eval(long long n, const double* __
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double p1 = p1f ? p1f[i] : P.p1, p2 = p2f ? p2f[i] : P.p2, x = psi[i];
     const double ks = Ks ? Ks[i] : Ks_s;
-    with_law_dd<MODEL>(P, Q, mat_at<MODEL>(mat, i), [&](auto law, const Phys<double>& Pc, const DDPhys& Qc) {
+    const unsigned mi = mat_at<MODEL>(mat, i);
+    if (DD && theta) theta[i] = dd_join(theta_x<MODEL>(x, p1, p2, mi, !p1f && !p2f, Q, P));
+    with_law_dd<MODEL>(P, Q, mi, [&](auto law, const Phys<double>& Pc, const DDPhys& Qc) {
       constexpr int ML = decltype(law)::value;
-      if (theta) theta[i] = DD ? theta_dd<ML>(x, p1, p2, Qc, Pc) : theta_only_d<ML>(x, p1, p2, Pc);
+      if (!DD && theta) theta[i] = theta_only_d<ML>(x, p1, p2, Pc);
       if (K) K[i] = DD ? cond_dd<ML>(x, p1, p2, ks, Qc, Pc) : cond_d<ML>(x, p1, p2, ks, Pc);
       return 0;
     });
@@ -613,22 +622,20 @@ __global__ void __launch_bounds__(256) k_mass_balance(Level<double> L, Geom G, B
     const dd p1 = L.p1 ? dd_split(L.p1[i]) : Q.p1, p2 = L.p2 ? dd_split(L.p2[i]) : Q.p2;
     const dd psi = dd_split(L.u[i]), pn = dd_split(psin[i]);
     const unsigned mi = mat_of<MODEL>(L, i);
-    dd th1, thn, hist, ps;
-    with_law_dd<MODEL>(P, Q, mi, [&](auto law, const Phys<double>& Pc, const DDPhys& Qc) {
-      constexpr int ML = decltype(law)::value;
-      th1 = th_new ? dd_split(th_new[i]) : theta_x<ML>(psi, p1, p2, Qc, Pc);
-      thn = th_n ? dd_split(th_n[i]) : theta_x<ML>(pn, p1, p2, Qc, Pc);
-      if (scheme == 1) {
-        hist = dd_mul(thn, hist_scale);
-        ps = pn;
-      } else {
-        const dd pm = dd_split(psinm1[i]);
-        const dd thm = th_nm1 ? dd_split(th_nm1[i]) : theta_x<ML>(pm, p1, p2, Qc, Pc);
-        hist = dd_mul(dd_sub(mk(4.0f * thn.hi, 4.0f * thn.lo), thm), hist_scale);
-        ps = Pc.lag ? pn : dd_sub(mk(2.0f * pn.hi, 2.0f * pn.lo), pm);
-      }
-      return 0;
-    });
+    dd hist, ps;
+    const double p1d = L.p1 ? L.p1[i] : P.p1, p2d = L.p2 ? L.p2[i] : P.p2;
+    const bool uniform = !L.p1 && !L.p2;
+    const dd th1 = th_new ? dd_split(th_new[i]) : theta_x<MODEL>(L.u[i], p1d, p2d, mi, uniform, Q, P);
+    const dd thn = th_n ? dd_split(th_n[i]) : theta_x<MODEL>(psin[i], p1d, p2d, mi, uniform, Q, P);
+    if (scheme == 1) {
+      hist = dd_mul(thn, hist_scale);
+      ps = pn;
+    } else {
+      const dd pm = dd_split(psinm1[i]);
+      const dd thm = th_nm1 ? dd_split(th_nm1[i]) : theta_x<MODEL>(psinm1[i], p1d, p2d, mi, uniform, Q, P);
+      hist = dd_mul(dd_sub(mk(4.0f * thn.hi, 4.0f * thn.lo), thm), hist_scale);
+      ps = P.lag ? pn : dd_sub(mk(2.0f * pn.hi, 2.0f * pn.lo), pm);
+    }
     const dd smax = L.smax ? dd_split(L.smax[i]) : mk(0.0f);
     dd cell = dd_sub(dd_mul(Q.a, th1), hist);
     cell = dd_add(cell, sink_x(psi, smax, Q));
