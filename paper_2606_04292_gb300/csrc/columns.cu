@@ -451,7 +451,7 @@ template <int MODEL>
 __global__ void __maxnreg__(72) k_columns(ColArgs A) {
   extern __shared__ float smem[];
   __shared__ Level<float> Ls[COL_MAXLEV];
-  __shared__ unsigned long long sm[33];
+  __shared__ unsigned long long sm[TEAM_WORDS];
   __shared__ double kb64[2];
   __shared__ ColShared S;
   __shared__ int s_col, s_nl;

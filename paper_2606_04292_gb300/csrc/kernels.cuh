@@ -505,9 +505,12 @@ __host__ __device__ inline bool nested_levels(int fn0, int fn1, int fn2, int cn0
 // over 16 SMs it takes the latency of one update, and the hardware barrier of
 // a cluster costs a fraction of a launch or of a grid-wide barrier.
 // ---------------------------------------------------------------------------
+constexpr int SEEN_CELLS = 64;         // the most coarsest cells that revisited() follows
+constexpr int TEAM_WORDS = 33 + SEEN_CELLS;
 struct BlockTeam {
   static constexpr bool splits = false;
-  unsigned long long* sm;              // 33 words
+  unsigned long long* sm;              // TEAM_WORDS words: block_max's, revisited()'s
+  __device__ unsigned long long* words() const { return sm; }
   __device__ unsigned rank() const { return threadIdx.x; }
   __device__ unsigned size() const { return blockDim.x; }
   __device__ void sync() const { __syncthreads(); }
@@ -517,7 +520,7 @@ struct BlockTeam {
 // Shared memory of a cluster team: block_max's words and two rotating rows of
 // one maximum per block.
 struct ClusterShared {
-  unsigned long long sm[33];
+  unsigned long long sm[TEAM_WORDS];
   unsigned long long part[2][CLUSTER_MAX];
 };
 
@@ -536,6 +539,7 @@ struct ClusterTeam {
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(ct));
     solo = nct == 1;
   }
+  __device__ unsigned long long* words() const { return sh->sm; }
   __device__ bool lead() const { return ct == 0; }
   __device__ unsigned rank() const {
     return solo ? threadIdx.x : (((threadIdx.x >> 5) * nct + ct) << 5) + (threadIdx.x & 31);
@@ -579,6 +583,7 @@ struct GridTeam {
   unsigned long long* sm;
   int round;
   bool solo;
+  __device__ unsigned long long* words() const { return sm; }
   __device__ bool lead() const { return blockIdx.x == 0; }
   __device__ unsigned rank() const { return solo ? threadIdx.x : blockIdx.x * blockDim.x + threadIdx.x; }
   __device__ unsigned size() const { return solo ? blockDim.x : gridDim.x * blockDim.x; }
@@ -656,6 +661,35 @@ __device__ __forceinline__ T team_defect(const Level<T>& L, const Phys<T>& P, bo
   return from_bits<T>(tm.max(mx));
 }
 
+// Whether the coarsest level's iterate is, bit for bit, the one of two sweeps
+// ago, kept in shared memory (first: only keeps it).  A sweep is a function of
+// the iterate, so from then on the sweeps alternate between two states, or
+// repeat one: the stop test has failed at both, and after an even number of
+// further sweeps the iterate is this one.  A defect at round-off need not fall
+// to crtol d0, and such a solve otherwise runs all its cmax sweeps.  GB300: two
+// steps of the Celia column 3.44 -> 2.44 ms, two-layer 256^2 13.25 -> 11.1, 4096
+// columns x 4 steps 38.0 -> 34.7, 513^2 strip 14.38 -> 14.04.
+// (Teams of several blocks that share the level, and levels of more than
+// SEEN_CELLS cells, do not look.)
+template <typename T, typename TM>
+__device__ __forceinline__ bool revisited(const Level<T>& L, bool first, TM& tm) {
+  if constexpr (TM::splits) {
+    if (!tm.solo) return false;
+  }
+  if (L.ncell > SEEN_CELLS) return false;
+  bool differs = first;
+  for (unsigned i = threadIdx.x; i < (unsigned)L.ncell; i += blockDim.x) {
+    const T v = L.u[i];
+    unsigned long long b;
+    if constexpr (sizeof(T) == 8) b = (unsigned long long)__double_as_longlong(v);
+    else b = __float_as_uint(v);
+    unsigned long long& kept = tm.words()[33 + i];
+    if (b != kept) differs = true;
+    kept = b;
+  }
+  return !__syncthreads_or(differs);
+}
+
 // Levels l0..nl-1 of one multigrid cycle by one team, with the recursion of
 // Section 3.2 unrolled: pre-smoothing, defect, restriction and the FAS right
 // side on the way down; gamma visits of each coarser level (1: V-cycle, 2:
@@ -675,7 +709,7 @@ __device__ __forceinline__ void team_cycle(const LV& lv, int l0, int nl, const P
   unsigned long long visits = 0;         // coarse visits done from each level, two bits a level (gamma <= 3)
   int l = l0, solo_at = -1;
   bool arrive = true;                    // at level l from above
-  int stage = DOWN, sweeps = 0, done = 0;
+  int stage = DOWN, sweeps = 0, done = 0, limit = 0;
   T d0 = T(0);
   for (;;) {
     bool finished = false;
@@ -695,6 +729,7 @@ __device__ __forceinline__ void team_cycle(const LV& lv, int l0, int nl, const P
       stage = l == nl - 1 ? COARSEST : DOWN;
       sweeps = stage == COARSEST ? (cmax > 1 ? 0 : 1) : nu1;
       done = 0;
+      limit = cmax;
     }
     if (!finished) {
       const Level<T>& F = lv.L(l);
@@ -703,10 +738,15 @@ __device__ __forceinline__ void team_cycle(const LV& lv, int l0, int nl, const P
       finished = true;
       if (stage == COARSEST) {
         done += sweeps;
-        if (done < cmax) {               // (the last sweep's defect would change nothing)
-          const T dn = team_defect<T, FORM, MODEL, TM>(F, P, false, tm);
-          if (done == 0) d0 = dn;
-          finished = done > 0 && !(dn > crtol * d0);
+        if (done < limit) {              // (the last sweep's defect would change nothing)
+          if (done > 1 && !(done & 1) && revisited<T>(F, done == 2, tm)) {
+            limit = done + ((limit - done) & 1);
+            finished = done == limit;
+          } else {
+            const T dn = team_defect<T, FORM, MODEL, TM>(F, P, false, tm);
+            if (done == 0) d0 = dn;
+            finished = done > 0 && !(dn > crtol * d0);
+          }
           sweeps = 1;
         }
         if (!finished) continue;
@@ -905,7 +945,7 @@ __global__ void __launch_bounds__(COOP_THREADS) k_coop_cycle(const Level<T>* __r
                                                              int tail_start, Phys<T> P, int nu1, int nu2, int cmax,
                                                              T crtol, int gamma, int gamma_levels,
                                                              unsigned long long* stats, unsigned long long* slots) {
-  __shared__ unsigned long long sm[33];
+  __shared__ unsigned long long sm[TEAM_WORDS];
   GridTeam tm{slots, sm, 0, false};
   if (tm.rank() == 0) slots[0] = slots[1] = slots[2] = 0ull;
   tm.sync();
