@@ -661,18 +661,23 @@ __device__ __forceinline__ T team_defect(const Level<T>& L, const Phys<T>& P, bo
   return from_bits<T>(tm.max(mx));
 }
 
-// Whether the coarsest level's iterate is, bit for bit, the one of two sweeps
-// ago, kept in shared memory (first: only keeps it).  A sweep is a function of
-// the iterate, so from then on the sweeps alternate between two states, or
-// repeat one: the stop test has failed at both, and after an even number of
-// further sweeps the iterate is this one.  A defect at round-off need not fall
-// to crtol d0, and such a solve otherwise runs all its cmax sweeps.  GB300: two
-// steps of the Celia column 3.44 -> 2.44 ms, two-layer 256^2 13.25 -> 11.1, 4096
-// columns x 4 steps 38.0 -> 34.7, 513^2 strip 14.38 -> 14.04.
-// (Teams of several blocks that share the level, and levels of more than
-// SEEN_CELLS cells, do not look.)
+// Whether the coarsest level's iterate is, bit for bit, the kept one (in shared
+// memory; first: there is none yet; keep: this one becomes it).  A sweep is a
+// function of the iterate, so from then on the sweeps repeat the states since
+// the kept one: the stop test has failed at all of them, and after a whole
+// number of such periods the iterate is this one.  Kept are the states after 2,
+// 4, 8, ... sweeps (Brent's cycle detection, BIT 20, 1980: any period is found
+// within twice the sweeps it took to begin).  A defect at round-off need not
+// fall to crtol d0, and such a solve otherwise runs all its cmax sweeps.
+// GB300, all sweeps / ended at a period of one or two (looked at every second
+// sweep) / at any: two steps of the Celia column 3.44 / 2.44 / 2.42 ms, two-layer
+// 256^2 13.3 / 11.1 / 10.4, 4096 columns x 4 steps 38.0 / 34.9 / 32.9, Gardner
+// 128^2 3.41 / 3.27 / 3.18, 8 served requests 9.94 / 9.82 / 9.55; keeping every
+// sixth or twelfth state 33.0 and 33.1 for the columns, 10.6 and 10.75 for the
+// two layers.  (Teams of several blocks that share the level, and levels of
+// more than SEEN_CELLS cells, do not look.)
 template <typename T, typename TM>
-__device__ __forceinline__ bool revisited(const Level<T>& L, bool first, TM& tm) {
+__device__ __forceinline__ bool revisited(const Level<T>& L, bool first, bool keep, TM& tm) {
   if constexpr (TM::splits) {
     if (!tm.solo) return false;
   }
@@ -685,7 +690,7 @@ __device__ __forceinline__ bool revisited(const Level<T>& L, bool first, TM& tm)
     else b = __float_as_uint(v);
     unsigned long long& kept = tm.words()[33 + i];
     if (b != kept) differs = true;
-    kept = b;
+    if (keep) kept = b;
   }
   return !__syncthreads_or(differs);
 }
@@ -739,8 +744,9 @@ __device__ __forceinline__ void team_cycle(const LV& lv, int l0, int nl, const P
       if (stage == COARSEST) {
         done += sweeps;
         if (done < limit) {              // (the last sweep's defect would change nothing)
-          if (done > 1 && !(done & 1) && revisited<T>(F, done == 2, tm)) {
-            limit = done + ((limit - done) & 1);
+          if (done > 1 && revisited<T>(F, done == 2, (done & (done - 1)) == 0, tm)) {
+            const int p = done - (1 << (31 - __clz(done - 1)));   // sweeps since the kept state
+            limit = done + (limit - done) % p;
             finished = done == limit;
           } else {
             const T dn = team_defect<T, FORM, MODEL, TM>(F, P, false, tm);
