@@ -2134,7 +2134,9 @@ richards_status richards_set_sink(richards_ctx* c, const richards_sink* k) {
   cudaStreamSynchronize(c->s);
   graphs_reset(c);
   if (const char* e = rich::sink_error(*k)) return fail(c, RICH_EINVAL, e);
+  const bool had_sink = c->sink.enabled != 0;
   c->sink = *k;
+  if (!k->enabled && had_sink && c->bc_set) return upload_views(c);   // (the device's views still hold the old one)
   return refresh_sink(c);
 }
 

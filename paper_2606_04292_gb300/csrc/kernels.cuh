@@ -630,7 +630,7 @@ __device__ __forceinline__ void team_sweep(const Level<T>& L, const Phys<T>& P, 
       }
       if (on) {
         if constexpr (TM::splits) {
-          if (L.smax) point_update<T, FORM, MODEL, 0, 1>(L, P, i, i0, i1, i2);
+          if (P.sink && L.smax) point_update<T, FORM, MODEL, 0, 1>(L, P, i, i0, i1, i2);
           else point_update<T, FORM, MODEL, 0, 0>(L, P, i, i0, i1, i2);
         } else {
           point_update<T, FORM, MODEL>(L, P, i, i0, i1, i2);
