@@ -367,9 +367,12 @@ __device__ __forceinline__ double cond_d(double psi, double p1, double p2, doubl
 //
 // The hardware's 1/x, log2 and 2^x are taken in their flush-to-zero forms:
 // the plain __fdividef, __logf, __expf wrap each in three to five
-// instructions that rescale subnormal operands, which no operand here needs
-// (a power below 1e-38 adds nothing to 1 + t), and a point update takes 16 of
-// them.  Reciprocals of per-cell values (1/(1 + t0)) are taken once per update.
+// instructions that rescale subnormal operands, and a point update takes 16 of
+// them.  A power of psi0 + x below 2^-126 adds nothing to 1 + t; one of psi0
+// is a factor that the increment multiplies by up to e^80, so dbase() keeps
+// it: heads whose power is flushed count as saturated, where the increment
+// comes from psi0 + x alone, and Gardner's e^(alpha psi0) takes the plain form.
+// Reciprocals of per-cell values (1/(1 + t0)) are taken once per update.
 // The point update is bound by instruction issue on big levels and by its own
 // instruction chain (~6 cycles per instruction of a lone warp) on small ones.
 // ---------------------------------------------------------------------------
@@ -429,13 +432,15 @@ template <int MODEL>
 __device__ __forceinline__ DBase dbase(float psi0, float p1, float p2) {
   DBase B;
   B.psi0 = psi0;
-  B.wet0 = !(psi0 < 0.0f);
+  // (heads nearer to saturation than the smallest normal number are: their
+  // reciprocal overflows)
+  B.wet0 = !(psi0 <= -1.17549435e-38f);
   B.inv_psi0 = B.wet0 ? 0.0f : rcp_a(psi0);
   B.a0 = B.b0 = B.c0 = B.r0 = 0.0f;
   B.m = MODEL == VANGENUCHTEN ? 1.0f - rcp_a(p2) : 0.0f;
   if (!B.wet0) {
     if (MODEL == GARDNER) {
-      B.a0 = exp_a(p1 * psi0);
+      B.a0 = __expf(p1 * psi0);
     } else if (MODEL == HAVERKAMP) {
       const float lu = fminf(p2 * log_a(-psi0), POW_EXP_MAX);   // h0^beta
       B.a0 = exp_a(lu);
@@ -448,6 +453,8 @@ __device__ __forceinline__ DBase dbase(float psi0, float p1, float p2) {
       B.c0 = exp_a(-m * B.b0);
       B.r0 = rcp_a(1.0f + B.a0);
     }
+    // a flushed power: theta(psi0) is theta_s to below 2^-126
+    if (MODEL != GARDNER) B.wet0 = B.a0 == 0.0f;
   }
   return B;
 }
