@@ -427,14 +427,15 @@ struct DBase {
 // turn into inf/inf; there theta = theta_r and theta' = 0 to far below FP32
 // resolution either way, so capping the exponent changes nothing else.
 constexpr float POW_EXP_MAX = 80.0f;
+// 2^-126: what is below it has no reciprocal here.  Heads nearer to
+// saturation count as saturated, a smaller coupling as none.
+constexpr float NORMAL_MIN = 1.17549435e-38f;
 
 template <int MODEL>
 __device__ __forceinline__ DBase dbase(float psi0, float p1, float p2) {
   DBase B;
   B.psi0 = psi0;
-  // (heads nearer to saturation than the smallest normal number are: their
-  // reciprocal overflows)
-  B.wet0 = !(psi0 <= -1.17549435e-38f);
+  B.wet0 = !(psi0 <= -NORMAL_MIN);
   B.inv_psi0 = B.wet0 ? 0.0f : rcp_a(psi0);
   B.a0 = B.b0 = B.c0 = B.r0 = 0.0f;
   B.m = MODEL == VANGENUCHTEN ? 1.0f - rcp_a(p2) : 0.0f;
@@ -464,7 +465,7 @@ __device__ __forceinline__ void dincr(const DBase& B, float x, float p1, float p
                                       float& Dth, float& dth) {
   const float ds = P.ts - P.tr;
   const float psi1 = B.psi0 + x;
-  const bool wet1 = !(psi1 < 0.0f);
+  const bool wet1 = !(psi1 <= -NORMAL_MIN);
   if (MODEL == GARDNER) {
     const float al = p1;
     if (!B.wet0) {
@@ -689,6 +690,9 @@ __device__ __forceinline__ bool is_zero(float a) { return a == 0.0f; }
 __device__ __forceinline__ bool is_zero(double a) { return (fl::dbits(a) << 1) == 0; }
 __device__ __forceinline__ bool above_zero(float a) { return a > 0.0f; }
 __device__ __forceinline__ bool above_zero(double a) { return (long long)fl::dbits(a) > 0 && !fl::is_nan(a); }
+// a coupling that can be divided by
+__device__ __forceinline__ bool couples(float a) { return a >= NORMAL_MIN; }
+__device__ __forceinline__ bool couples(double a) { return above_zero(a); }
 __device__ __forceinline__ float clamp_to(float x, float lo, float hi) { return x < lo ? lo : (x > hi ? hi : x); }
 __device__ __forceinline__ double clamp_to(double x, double lo, double hi) {
   if (fl::is_nan(x) || fl::is_nan(lo) || fl::is_nan(hi)) return x;
@@ -699,7 +703,7 @@ __device__ __forceinline__ double clamp_to(double x, double lo, double hi) {
 template <typename T, int FORM, int MODEL, int NK = 0, int SINK = -1>
 __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T smax, const Phys<T>& P,
                                          const LawCell<FORM == FORM_DIRECT ? MODEL : -1>& law) {
-  if (!above_zero(cc)) {
+  if (!couples(cc)) {
     // no coupling and no shift (c = 0): shift kappa (x - x0), kappa = 1e-6 a,
     // which keeps the root and provides the bracket
     const T k = T(1e-6) * P.a;

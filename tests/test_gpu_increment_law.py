@@ -1,6 +1,7 @@
-"""The FP32 increment law where a power of the frozen state leaves FP32's
-normal range (needs a GPU): heads close to saturation under a steep law, and
-dry Gardner soils whose conductivity has all but vanished.
+"""The FP32 increment law where a power of the frozen state, or the coupling
+to the neighbours, leaves FP32's normal range (needs a GPU): heads close to
+saturation under a steep law, and dry Gardner soils whose conductivity has all
+but vanished.
 
 One outer correction of a four-cell column, whose inner problem is solved to
 its round-off.  The correction law is good to ~2e-5 of the storage change (an
@@ -52,6 +53,15 @@ def test_drainage_from_just_below_saturation(law, p1, p2, psi0):
 @pytest.mark.parametrize("psi0", [-86.0, -88.0, -90.0, -91.0])
 def test_infiltration_into_a_dry_gardner_soil(psi0):
     soil = W._soil(W.GARDNER, Ks=100.0, theta_s=0.4, theta_r=0.1, p1=1.0)
+    bc = W._bc([W.NOFLUX, W.FLUX], [0.0, 1e-6])
+    r = _drop(soil, bc, psi0, 1.0)
+    assert r <= 1e-3, r
+
+
+@pytest.mark.parametrize("psi0", [-79.0, -81.0, -86.0, -90.0, -91.0])
+def test_infiltration_into_a_gardner_soil_that_hardly_conducts(psi0):
+    """K / h^2 below 2^-126 (1e-5 e^-79 = 5e-40) and not yet 0 in FP32."""
+    soil = W._soil(W.GARDNER, Ks=1e-5, theta_s=0.4, theta_r=0.1, p1=1.0)
     bc = W._bc([W.NOFLUX, W.FLUX], [0.0, 1e-6])
     r = _drop(soil, bc, psi0, 1.0)
     assert r <= 1e-3, r
