@@ -430,7 +430,7 @@ __device__ __forceinline__ double cond_dd(double psi, double p1, double p2, doub
   return dd_join(cond_x<MODEL>(dd_split(psi), dd_split(p1), dd_split(p2), dd_split(Ks), Q, P));
 }
 
-// Feddes sink S = smax alpha_F(psi) (same pieces as feddes()); thresholds
+// Feddes sink S = smax alpha_F(psi) (same pieces as feddes_piece()); thresholds
 // are compared in float-float, so a psi within 2^-46 of a kink may take the
 // neighbouring piece, where alpha_F agrees to that order (it is continuous)
 __device__ __forceinline__ dd sink_x(dd psi, dd smax, const DDPhys& Q) {

@@ -677,8 +677,8 @@ __global__ void __launch_bounds__(256) k_mass_balance(Level<double> L, Geom G, B
       return 0;
     });
     const float smf = dd_float(smax);
-    float sa = 0.0f, sda = 0.0f;
-    if (Pf.sink && smf > 0.0f) feddes(psif, Pf, sa, sda);
+    float sda = 0.0f;
+    if (Pf.sink && smf > 0.0f) feddes_piece(psif, Pf, sda);
     dmin = fminf(dmin, Pf.a * dth + sda * smf + Pf.xi);
   }
   acc = warp_sum_dd(acc);
@@ -779,8 +779,8 @@ __global__ void __launch_bounds__(256) k_mass_balance64(Level<double> L, Geom G,
       return 0;
     });
     const float smf = (float)smax;
-    float sa = 0.0f, sda = 0.0f;
-    if (Pf.sink && smf > 0.0f) feddes(psif, Pf, sa, sda);
+    float sda = 0.0f;
+    if (Pf.sink && smf > 0.0f) feddes_piece(psif, Pf, sda);
     dmin = fminf(dmin, Pf.a * dth + sda * smf + Pf.xi);
   }
   for (int o = 16; o > 0; o >>= 1) {
