@@ -130,8 +130,8 @@ void batch32(int op, int nk, const BJob32* table, const BList& list, int color, 
 void batch_tail32(const BJob32* table, const BList& list, int blocks, int nu1, int nu2, int cmax, float crtol, int gamma,
                   int gamma_levels, cudaStream_t s) {
   if (list.n <= 0) return;
-  launch_cluster(k_tail_batch32, blocks, list.n, TAIL_THREADS, s, table, list, nu1, nu2, cmax, crtol, gamma,
-                 gamma_levels);
+  launch_cluster<k_tail_batch32>(blocks, list.n, TAIL_THREADS, s, table, list, nu1, nu2, cmax, crtol, gamma,
+                                 gamma_levels);
 }
 
 }  // namespace rich

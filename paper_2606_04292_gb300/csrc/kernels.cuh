@@ -988,32 +988,58 @@ inline Launch3 launch3(int nx, int n1, int n2, int bx_force = 0) {
   return L;
 }
 
-// launches `clusters` clusters of `blocks` thread blocks; clusters of more
-// than 8 blocks need the kernel's consent (a non-portable size), and a device
-// that cannot place such a cluster takes the next smaller power of two
-template <typename... KA, typename... A>
-inline cudaError_t launch_cluster(void (*kern)(KA...), int blocks, int clusters, int threads, cudaStream_t s, A... args) {
+// what the device says of one kernel's clusters (cluster_fit.h)
+template <auto KERN>
+struct ClusterQuery {
+  int threads;
+  bool pending() const { return cudaPeekAtLastError() != cudaSuccess; }
+  bool consent() const {
+    return cudaFuncSetAttribute(KERN, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  }
+  int held(int blocks) const {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    return cudaOccupancyMaxActiveClusters(&n, KERN, &cfg) == cudaSuccess ? n : -1;
+  }
+  void clear() const { cudaGetLastError(); }
+};
+template <auto KERN>
+inline int cluster_blocks(int blocks, int clusters, int threads) {
+  static ClusterFit fits[16];          // by device; a device beyond them is asked every time
+  ClusterFit asked;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return fit_blocks(dev >= 0 && dev < 16 ? fits[dev] : asked, blocks, clusters, ClusterQuery<KERN>{threads});
+}
+
+// launches `clusters` clusters of `blocks` thread blocks each, or of the next
+// smaller power of two that the device can place
+template <auto KERN, typename... KA, typename... A>
+inline cudaError_t launch_cluster_as(void (*kern)(KA...), int blocks, int clusters, int threads, cudaStream_t s,
+                                     A... args) {
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cluster_blocks<KERN>(blocks, 1, threads);
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(at.val.clusterDim.x * clusters);
   cfg.blockDim = dim3(threads);
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  if (blocks > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-    cudaGetLastError();
-    blocks = 8;
-  }
-  for (;; blocks >>= 1) {
-    at.val.clusterDim.x = blocks;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.gridDim = dim3(blocks * clusters);
-    if (blocks <= 8) break;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) break;
-    cudaGetLastError();
-  }
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KA>(args)...);
+}
+template <auto KERN, typename... A>
+inline cudaError_t launch_cluster(int blocks, int clusters, int threads, cudaStream_t s, A... args) {
+  return launch_cluster_as<KERN>(KERN, blocks, clusters, threads, s, args...);
 }
 
 // host: calls fn(LawTag<model>{}) for a runtime law (COMPOSITE included)
@@ -1148,7 +1174,7 @@ struct Dispatch {
                          const double* const* kb, cudaStream_t s) {
     FaceSource src{};
     for (int f = 0; kb && f < 6; ++f) src.kb[f] = kb[f];
-    launch_cluster(k_team_setup<T>, blocks, 1, TAIL_THREADS, s, dLs, dXs, nl, ts, psi0, src);
+    launch_cluster<k_team_setup<T>>(blocks, 1, TAIL_THREADS, s, dLs, dXs, nl, ts, psi0, src);
   }
   // the cooperative coarse cycle: the most blocks that can be co-resident
   static int coop_max_blocks(int model) {
@@ -1181,8 +1207,9 @@ struct Dispatch {
                    int model, int nu1, int nu2, int cmax, T crtol, int gamma, int gamma_levels,
                    unsigned long long* stats, int ordering, cudaStream_t s) {
     by_model(model, [&](auto m) {
-      launch_cluster(k_tail<T, FORM, decltype(m)::value>, ts.blocks, 1, TAIL_THREADS, s, dLs, dXs, l0, nl,
-                     ts.tail_start, ts.handoff, P, nu1, nu2, cmax, crtol, gamma, gamma_levels, stats, ordering);
+      launch_cluster<k_tail<T, FORM, decltype(m)::value>>(ts.blocks, 1, TAIL_THREADS, s, dLs, dXs, l0, nl,
+                                                          ts.tail_start, ts.handoff, P, nu1, nu2, cmax, crtol, gamma,
+                                                          gamma_levels, stats, ordering);
     });
   }
 };

@@ -5,6 +5,7 @@
 
 #include "richards.h"
 
+#include "cluster_fit.h"
 #include "ddmath.cuh"
 #include "device.cuh"
 
@@ -28,7 +29,6 @@ struct Geom {
 // How the coarse tail runs: one cluster of `blocks` blocks; levels from
 // `handoff` on by its first block alone; transfers below `tail_start` as the
 // grid kernels take them (nested formulas), from it on through the tables.
-constexpr int CLUSTER_MAX = 16;
 struct TeamShape {
   int blocks, handoff, tail_start;
 };

@@ -420,7 +420,7 @@ long long build_plan(const richards_grid* grid, const richards_soil* soil, const
 
 void launch_plan(const NaPlan& p, cudaStream_t s) {
   by_model(p.model, [&](auto m) {
-    launch_cluster(k_small_step<decltype(m)::value>, p.blocks, 1, TAIL_THREADS, s, p);
+    launch_cluster<k_small_step<decltype(m)::value>>(p.blocks, 1, TAIL_THREADS, s, p);
   });
 }
 
