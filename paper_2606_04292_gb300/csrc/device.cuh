@@ -568,30 +568,33 @@ __device__ __forceinline__ int feddes_piece(T psi, const Phys<T>& P, T& da) {
   da = P.r34;
   return 3;
 }
-// alpha_F at psi on piece k
-template <typename T>
-__device__ __forceinline__ T feddes_value(T psi, int k, const Phys<T>& P) {
-  if (k == 1) return ramp(P.h1 - psi, P.h1 - P.h2, P.r12);
-  if (k == 3) return ramp(psi - P.h4, P.h3 - P.h4, P.r34);
-  return k == 2 ? T(1) : T(0);
-}
-
 // alpha_F(psi1) - alpha_F(psi0), on pieces k1 and k0.  A correction seldom
 // crosses a kink, so this is a call (by value: a reference would put the
 // physics in memory): inlined, the two ramps at every update cost the served
 // mix 6% (8 requests 8.66 -> 9.16 ms).
 static __device__ __noinline__ float feddes_jump(float psi0, int k0, float psi1, int k1, float h1, float h2, float h3,
                                                  float h4, float r12, float r34) {
-  Phys<float> P;
-  P.h1 = h1; P.h2 = h2; P.h3 = h3; P.h4 = h4;
-  P.r12 = r12; P.r34 = r34;
-  return feddes_value(psi1, k1, P) - feddes_value(psi0, k0, P);
+  auto value = [=](float psi, int k) {
+    if (k == 1) return ramp(h1 - psi, h1 - h2, r12);
+    if (k == 3) return ramp(psi - h4, h3 - h4, r34);
+    return k == 2 ? 1.0f : 0.0f;
+  };
+  return value(psi1, k1) - value(psi0, k0);
 }
 
-template <typename T>
-__device__ __forceinline__ void sink_direct(T psi, T smax, const Phys<T>& P, T& S, T& dS) {
-  T a = T(0), da = T(0);
-  if (P.sink && smax > T(0)) a = feddes_value(psi, feddes_piece(psi, P, da), P);
+// alpha_F in FP64 on a ramp (a call as well: the FP64 operations of both ramps
+// would otherwise issue in every update, with or without a sink)
+static __device__ __noinline__ double feddes_ramp(double psi, int k, double h1, double h2, double h3, double h4,
+                                                  double r12, double r34) {
+  return k == 1 ? ramp(h1 - psi, h1 - h2, r12) : ramp(psi - h4, h3 - h4, r34);
+}
+__device__ __forceinline__ void sink_direct(double psi, double smax, const Phys<double>& P, double& S, double& dS) {
+  double a = 0.0, da = 0.0;
+  if (P.sink && smax > 0.0) {
+    const int k = feddes_piece(psi, P, da);
+    a = k == 2 ? 1.0 : 0.0;
+    if (k & 1) a = feddes_ramp(psi, k, P.h1, P.h2, P.h3, P.h4, P.r12, P.r34);
+  }
   S = a * smax;
   dS = da * smax;
 }
