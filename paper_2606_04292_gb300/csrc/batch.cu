@@ -127,6 +127,15 @@ void batch32(int op, int nk, const BJob32* table, const BList& list, int color, 
   }
 }
 
+// (clusters of the biggest size up to `blocks` of which the GPU holds all the
+// listed tails at once: 7 of 16 blocks, 15 of 8, 36 of 4, 76 of 2.  In a
+// second wave the last tails would wait for the first ones' whole cycles,
+// most of it latency on idle SMs.  8 tails of 16 blocks / 8 at once: Gardner
+// 64^2 2.48 / 1.72 ms a step, drainage 33^3 8.51 / 6.31; 64 tails of 16 / 4 /
+// 2 blocks: 13.6 / 7.1 / 6.4 and 51.9 / 33.0 / 30.4 (10.2 and 42.0 with one
+// block each and the same levels above them as stage launches).  A smaller
+// request in a bigger one's launch leaves its other blocks at a barrier, which
+// costs nothing while all are placed.)
 void batch_tail32(const BJob32* table, const BList& list, int blocks, int nu1, int nu2, int cmax, float crtol, int gamma,
                   int gamma_levels, cudaStream_t s) {
   if (list.n <= 0) return;

@@ -1021,14 +1021,14 @@ inline int cluster_blocks(int blocks, int clusters, int threads) {
 }
 
 // launches `clusters` clusters of `blocks` thread blocks each, or of the next
-// smaller power of two that the device can place
+// smaller power of two of which the device holds them all at once
 template <auto KERN, typename... KA, typename... A>
 inline cudaError_t launch_cluster_as(void (*kern)(KA...), int blocks, int clusters, int threads, cudaStream_t s,
                                      A... args) {
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cluster_blocks<KERN>(blocks, 1, threads);
+  at.val.clusterDim.x = cluster_blocks<KERN>(blocks, clusters, threads);
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.gridDim = dim3(at.val.clusterDim.x * clusters);
   cfg.blockDim = dim3(threads);
