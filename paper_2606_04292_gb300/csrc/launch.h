@@ -56,8 +56,13 @@ inline TeamShape team_shape(const long long* cells, int l0, int nl, int tail_sta
 // (~5 us in a graph).  FP64: 65^2 in (257^2 strip 3.08 -> 2.92 ms), 24^3 out
 // (96^3 21.0 -> 21.6 ms with it).  FP32: 2-d levels to 128^2 (two-layer 256^2
 // 15.8 -> 14.5 ms), 3-d ones only to 16384 cells (32^3: 256^3 step 1.5% slower
-// with it).  Batched contexts: 33^3 too, so that the mix leaves its grid
-// stages together (8 requests 9.1 -> 7.6 ms).
+// with it).  Batched contexts: 66000, where the stages are launched directly
+// and the tails of all requests together fill the GPU (batch_tail32).  A step
+// of n requests with level 1 of so many cells in stage launches / in clusters:
+// 26^3 12 requests 13.1 / 11.8 ms, 64: 81.6 / 69.9; 33^3 8: 18.9 / 18.0, 32:
+// 74.0 / 65.9; 36^3 8: 20.8 / 20.2, 32: 87.4 / 78.1; 40^3 1: 7.2 / 7.75, 4:
+// 14.2 / 13.7, 16: 50.2 / 47.3; 2-d 129^2 1: 0.90 / 0.86, 64: 8.5 / 8.1, 255^2
+// 1: 0.94 / 0.96, 8: 2.31 / 2.35, 32: 7.55 / 7.41.
 template <typename T>
 inline long long cluster_cells(int dim, bool batched = false) {
   return sizeof(T) == 8 ? 4608 : batched ? 66000 : dim < 3 ? 32768 : 16384;

@@ -57,3 +57,14 @@ def test_any_number_of_requests():
     alone = _alone(kinds)
     for n in (1, 7, 8, 15, 16, 36, 37, 64, 77):
         _check([kinds[k % len(kinds)] for k in range(n)], alone)
+
+
+@pytest.mark.parametrize("n", [2, 9, 18])
+@pytest.mark.parametrize("sizes", [[(80, 80, 79), (82, 81, 82)], [(514, 510), (514, 514)]])
+def test_levels_on_both_sides_of_the_clusters_limit(n, sizes):
+    """Level 1 just below and just above the 66000 cells that clusters take."""
+    probs = [W.random_problem(len(m), m, W.VANGENUCHTEN, 6, **OPTS) for m in sizes]
+    for p in probs:
+        p["psi0"] = 0.2 * p["psi0"] - 0.5
+    alone = _alone(probs)
+    _check([probs[k % 2] for k in range(n)], alone)
