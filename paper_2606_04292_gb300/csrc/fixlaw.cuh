@@ -30,13 +30,12 @@
 // log2(1 + 2^-|t|) and 1 - 2^-u keep their relative accuracy for small
 // arguments: there the series multiplies the normalised argument itself.
 //
-// Errors over 4e6 random soils and heads (alpha 0.3-5, n 1.05-5.5, l -2-3, h
-// 1e-6-150) against 113-bit values, in ulps of the result, largest / rms; in
-// brackets the same formulas with a correctly rounded-to-an-ulp FP64 exp and
-// log, whose exponent carries the rounding of n log(alpha h):
-//   van Genuchten Se 1.0/0.31 (63/2.1), slope 1.7/0.53 (96/6.7), K/Ks
-//   2.1/0.34 (245/5.9); Haverkamp Se 0.9/0.29, slope 1.6/0.50; Gardner
-//   0.7/0.29.
+// Errors over 4e6 random soils and heads (alpha 0.3-5, n 1.05-5.5, l -2-2.5, h
+// 1e-6-150; Haverkamp beta 0.5-5) against 64-bit significands, in ulps of the
+// result, largest / rms: van Genuchten Se 1.1/0.30, slope 1.8/0.53, K/Ks
+// 2.1/0.35; Haverkamp Se 0.9/0.27, slope 1.7/0.48, K/Ks 0.8/0.27; Gardner
+// 0.8/0.30.  (In FP64 the exponent carries the rounding of n log(alpha h): tens
+// of ulps.)
 // Measured against the table-driven FP64 functions (GB300): theta and K of
 // 128^3 cells 840 -> 118 us; preparation of a 256^3 step 6.23 -> 1.38 ms; its
 // FP64 outer defect 3.96 -> 1.66 ms (the stencil's FP64 remains); an FP64
@@ -45,14 +44,21 @@
 // Arguments outside the ranges the integers hold (a head or alpha outside
 // 2^+-100, an exponent |t| above 120, n outside [1/32, 16): the 2^-57 of
 // log2 is carried into t n times) take the FP64 functions of fp64math.cuh (slow_* in device.cuh).
+//
+// A host compiler takes this file as well (the laws' integer arithmetic is
+// tested so, without a device).
 #pragma once
 
-#ifdef __CUDACC__
 #include <cmath>
+#include <cstring>
 
+#ifdef __CUDACC__
 #include "fp64math.cuh"
 #define RICH_FD __device__ __forceinline__
 #else
+#define __device__
+#include "fp64_tables.h"
+#undef __device__
 #define RICH_FD inline
 #endif
 
@@ -70,6 +76,23 @@ RICH_FD int clz64(u64 a) { return __clzll((long long)a); }
 RICH_FD u64 dbits(double x) { return (u64)__double_as_longlong(x); }
 RICH_FD double bitsd(u64 b) { return __longlong_as_double((long long)b); }
 RICH_FD u32 rcp_bits(u32 b) { return __float_as_uint(__frcp_rn(__uint_as_float(b))); }
+static __device__ __noinline__ double slow_div(double a, double b) { return a / b; }
+#else
+template <typename B, typename A>
+inline B bit_copy(A a) {
+  static_assert(sizeof(A) == sizeof(B), "same size");
+  B b;
+  std::memcpy(&b, &a, sizeof b);
+  return b;
+}
+inline u32 mulhi32(u32 a, u32 b) { return (u32)(((u64)a * b) >> 32); }
+inline u64 mulhi_exact(u64 a, u64 b) { return (u64)(((unsigned __int128)a * b) >> 64); }
+inline int clz64(u64 a) { return a ? __builtin_clzll(a) : 64; }
+inline u64 dbits(double x) { return bit_copy<u64>(x); }
+inline double bitsd(u64 b) { return bit_copy<double>(b); }
+inline u32 rcp_bits(u32 b) { return bit_copy<u32>(1.0f / bit_copy<float>(b)); }
+inline double slow_div(double a, double b) { return a / b; }
+using std::fma;
 #endif
 
 // high word of a 64 x 64-bit product, at most 3 below the exact one (the
@@ -266,7 +289,6 @@ RICH_FD Prep prep(double p1, double p2) {
 
 // The same on the host, for parameters known before a launch (a uniform soil,
 // a material): log2 in extended precision, the reciprocal by exact division.
-#ifdef __CUDACC__
 inline Prep host_prep(bool vg, double p1, double p2) {
   Prep q{0, 0, 0, false};
   const double ap = std::fabs(p1);
@@ -283,7 +305,6 @@ inline Prep host_prep(bool vg, double p1, double p2) {
   q.ok = true;
   return q;
 }
-#endif
 
 // theta's exponent: Se = 2^-u (scale 2^56)
 template <bool VG>
@@ -443,8 +464,11 @@ RICH_FD bool is_nan(double x) { return (dbits(x) << 1) > 0xffe0000000000000ull; 
 
 // A divisor b and its reciprocal, rounded to nearest from 61 bits (integer
 // Newton-Raphson).  div(a) is Markstein's quotient (IBM J. Res. Dev. 34,
-// 1990): q = a y, then q + (a - b q) y, the correctly rounded a/b.  Exponents
-// near the ends of the range, where a - b q could leave it, divide plainly.
+// 1990): q = a y, then q + (a - b q) y.  It is the correctly rounded a/b for a
+// correctly rounded y; this y can be the other neighbour (about once in 1200
+// times), where correctness is tested and not proven: none of 2e8 random
+// quotients differed from a/b.  Exponents near the ends of the range, where
+// a - b q could leave it, divide plainly.
 struct Divisor {
   double b, y;
   int e;
@@ -464,14 +488,11 @@ RICH_FD bool div_ok(double a, const Divisor& d) {
   const u64 k = dbits(a) << 1;
   return (u32)(d.e - 623) < 800u && ((u32)((int)(k >> 53) - 623) < 800u || k == 0);
 }
-#ifdef __CUDACC__
-static __device__ __noinline__ double slow_div(double a, double b) { return a / b; }
 RICH_FD double div(double a, const Divisor& d) {
   if (!div_ok(a, d)) return slow_div(a, d.b);
   const double q = a * d.y;
   return fma(fma(-q, d.b, a), d.y, q);
 }
-#endif
 
 }  // namespace fl
 }  // namespace rich
