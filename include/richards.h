@@ -356,7 +356,7 @@ richards_status richards_set_launch(richards_ctx *ctx, int level, int planes, in
    cells, down to the coarsest, run as one cooperative launch per visit --
    every block of the grid walks the cycle, with a grid barrier between
    stages instead of a launch per stage, and block 0 alone takes the levels
-   of the single-block tail.  Same values as the stage launches.  Off (0) by
+   of the coarse tail.  Same values as the stage launches.  Off (0) by
    default: on the 256^3 drainage the grid barriers cost more than the
    graph-replayed launches they replace.  EINVAL for a negative size. */
 richards_status richards_set_coop(richards_ctx *ctx, long long max_cells);
@@ -507,8 +507,9 @@ int richards_profile_read(richards_ctx *ctx, richards_kernel_stat *out, int max)
  * One implicit step (eq. fully-bdf1 or the BDF2 reading, solved by the FAS
  * cycles of Section 3.2 with the point update of eq. point-update: the same
  * arithmetic as richards_step in FP64 mode) of a grid with at most
- * RICHARDS_NOALLOC_MAX_CELLS cells, run in a single thread block.  psi_n, psi_prev (nullable: BDF1 is used) and psi_out are device
- * arrays of ncell doubles; psi_out may alias psi_n or psi_prev (both are
+ * RICHARDS_NOALLOC_MAX_CELLS cells, run in a single launch (one
+ * cluster of thread blocks).  psi_n, psi_prev (nullable: BDF1 is used) and
+ * psi_out are device arrays of ncell doubles; psi_out may alias psi_n or psi_prev (both are
  * read before anything is written).  In this call the optional soil fields
  * (Ks_field, p1_field, p2_field) and boundary fields (value_field,
  * mask_field) are DEVICE pointers.  The soil, boundary and sink parameters

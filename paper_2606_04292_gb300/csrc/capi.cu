@@ -28,7 +28,7 @@ using rich::law_error;
 namespace {
 
 constexpr int MAXLEV = 24;
-constexpr int NSCRATCH = 72;   // norm slots + statistics (32..63: the single-block step's; 64..66: the
+constexpr int NSCRATCH = 72;   // norm slots + statistics (32..63: the small-grid step's; 64..66: the
                                // cooperative cycle's reductions; 67..71: the inner-loop graph's control)
 // Levels of at most this many cells run as one cooperative launch: 0, off by
 // default -- on the 256^3 drainage its grid barriers cost more than the
@@ -163,8 +163,8 @@ struct richards_ctx {
   // richards_set_launch; 0 = the defaults): cells per thread along z of the
   // half-sweeps, their block x-size, the defect kernel's block x-size
   int tune_planes[MAXLEV] = {}, tune_bx[MAXLEV] = {}, tune_rbx[MAXLEV] = {};
-  // FP32 inner cycles: levels from coop_start down to the single-block tail
-  // run as one cooperative launch (MAXLEV: none); its grid size
+  // FP32 inner cycles: levels from coop_start down to the coarse tail run
+  // as one cooperative launch (MAXLEV: none); its grid size
   int coop_start = MAXLEV, coop_blocks = 0;
   // batcher progress (richards_batcher_step / _advance); reset by any call
   // that prepares a step or changes the problem
@@ -633,7 +633,7 @@ int team_start(const richards_ctx* c, bool batched = false) {
 // ------------------------------------------------------------------------
 // One V-cycle (Section 3.2, steps 1-7 with the coarse solve replaced by the
 // recursion) from level l: grid kernels down to the coarse tail, which runs
-// in one thread block.
+// in one cluster of thread blocks.
 // ------------------------------------------------------------------------
 // d_ready: as for vcycle32 (nu1 = 0 and the finest defect already current)
 void vcycle64(richards_ctx* c, int l, bool d_ready = false) {
@@ -2309,8 +2309,8 @@ richards_status richards_step(richards_ctx* c, double dt, int scheme, richards_s
 }
 
 // A grid of at most RICHARDS_NOALLOC_MAX_CELLS cells in FP64 (no FMG start):
-// the step -- preparation, stop tests and every cycle -- runs in one thread
-// block on the context's own hierarchy, one launch and one synchronisation
+// the step -- preparation, stop tests and every cycle -- runs in one
+// cluster of thread blocks on the context's own hierarchy, one launch and one synchronisation
 // instead of a launch per stage and a host round trip per cycle (the same
 // arithmetic as the grid path: apply_N, the point update and the transfers
 // are shared; layered soils included).
@@ -2351,7 +2351,7 @@ static richards_status step_small(richards_ctx* c, double dt, int scheme, richar
   if (rich::small_step(&c->grid, &soil, &bc, &c->sink, &c->opts, dt, scheme, c->psi_n,
                        scheme == 2 ? c->psi_nm1 : nullptr, F.u, (double*)(c->scratch + 32), &cx, c->opts.ordering,
                        stats, c->s) != RICH_OK)
-    return fail(c, RICH_ECUDA, "single-block step failed");
+    return fail(c, RICH_ECUDA, "small-grid step failed");
   const double r = stats[2];
   const richards_status st = (richards_status)(int)stats[3];
   if (info) {

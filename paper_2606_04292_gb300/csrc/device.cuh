@@ -1,7 +1,7 @@
 // Device building blocks of the NGS-FAS solver: constitutive laws, the
 // conservative 7-point (2d+1) stencil, the bracketed Newton point update,
 // the nonlinear defect, and the transfer operators.  Grid kernels and the
-// single-block coarse tail both call these functions.
+// coarse tail both call these functions.
 #pragma once
 
 #include <cuda_runtime.h>

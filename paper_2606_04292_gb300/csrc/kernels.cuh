@@ -1,4 +1,4 @@
-// Grid kernels of one V-cycle level and the single-block coarse tail.
+// Grid kernels of one V-cycle level and the coarse tail (one cluster of blocks).
 // Included by the FP64 and FP32 translation units, which instantiate them.
 #pragma once
 
@@ -943,7 +943,7 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_team_setup(const Level<T>* 
 
 // The coarse levels of a big grid as one cooperative launch, a grid barrier
 // between phases instead of a launch per stage; block 0 alone takes the
-// single-block tail's levels.  slots: three global words for the grid
+// coarse tail's levels.  slots: three global words for the grid
 // reductions; stats: the update count
 template <typename T, int FORM, int MODEL>
 __global__ void __launch_bounds__(COOP_THREADS) k_coop_cycle(const Level<T>* __restrict__ Ls,

@@ -107,7 +107,7 @@ void team_setup32(const Level<float>* dLs, const Xfer<float>* dXs, int nl, int t
 void team_setup64(const Level<double>* dLs, const Xfer<double>* dXs, int nl, int ts, int blocks, cudaStream_t s);
 void sweep_lex32(const Level<float>& L, const Phys<float>& P, int model, cudaStream_t s);
 // the cycle from level l0 down as one cooperative launch of `blocks` blocks
-// (levels from tail_start on take the single-block tail's transfers); slots:
+// (levels from tail_start on take the coarse tail's transfers); slots:
 // three device words for its reductions; stats: its update count
 constexpr int COOP_THREADS = 256;
 int coop_max_blocks32(int model);
@@ -231,8 +231,9 @@ void batch_tail32(const BJob32* table, const BList& list, int blocks, int nu1, i
 }  // namespace rich
 
 // ---------------------------------------------------------------------------
-// One FP64 step of a small grid in a single thread block (noalloc.cu): the
-// allocation-free entry point and contexts whose grid fits one block use it.
+// One FP64 step of a small grid in one cluster of thread blocks (noalloc.cu):
+// the allocation-free entry point and contexts of at most
+// RICHARDS_NOALLOC_MAX_CELLS cells use it.
 // ---------------------------------------------------------------------------
 namespace rich {
 
