@@ -507,10 +507,10 @@ int richards_profile_read(richards_ctx *ctx, richards_kernel_stat *out, int max)
  * One implicit step (eq. fully-bdf1 or the BDF2 reading, solved by the FAS
  * cycles of Section 3.2 with the point update of eq. point-update: the same
  * arithmetic as richards_step in FP64 mode) of a grid with at most
- * RICHARDS_NOALLOC_MAX_CELLS cells, run in a single launch (one
- * cluster of thread blocks).  psi_n, psi_prev (nullable: BDF1 is used) and
- * psi_out are device arrays of ncell doubles; psi_out may alias psi_n or psi_prev (both are
- * read before anything is written).  In this call the optional soil fields
+ * RICHARDS_NOALLOC_MAX_CELLS cells, run in a single launch (one cluster of
+ * thread blocks).  psi_n, psi_prev (nullable: BDF1 is used) and psi_out are
+ * device arrays of ncell doubles; psi_out may alias psi_n or psi_prev (both
+ * are read before anything is written).  In this call the optional soil fields
  * (Ks_field, p1_field, p2_field) and boundary fields (value_field,
  * mask_field) are DEVICE pointers.  The soil, boundary and sink parameters
  * are checked as by richards_set_soil / set_bc / set_sink (fields

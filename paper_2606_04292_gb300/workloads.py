@@ -293,9 +293,10 @@ def drainage_3d(n=256, dt=300.0, nsteps=50, seed_ks=3, seed_vg=4, **optkw):
     # against 33.3 ms at 256^3, when it was measured).  Each FP32 inner solve
     # reduces its defect 5e3-fold (two or three outer corrections reach tol
     # 1e-8), and levels of up to 512 cells run in the coarse tail.  One
-    # safeguarded Newton step per point update gives the same cycles per step here as two in 8% less time.  Coarsening
-    # stops at 8^3: as many cycles as with a 4^3 level below it, 6% less
-    # time; one sweep there and an inner target of 2e-4 save another 2%.
+    # safeguarded Newton step per point update gives the same cycles per step
+    # here as two in 8% less time.  Coarsening stops at 8^3: as many cycles as
+    # with a 4^3 level below it, 6% less time; one sweep there and an inner
+    # target of 2e-4 save another 2%.
     opts = default_opts(kappa_mode=0, kappa=0.0, xi=0.0, precision=1, cycle_gamma=2, gamma_levels=2,
                         nu1=0, nu2=2, coarse_max_sweeps=1, coarsest_max_n=8, inner_rtol=2e-4, tail_cells=512,
                         newton_iters=1)
