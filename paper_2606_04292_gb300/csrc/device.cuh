@@ -427,6 +427,7 @@ struct DBase {
 // turn into inf/inf; there theta = theta_r and theta' = 0 to far below FP32
 // resolution either way, so capping the exponent changes nothing else.
 constexpr float POW_EXP_MAX = 80.0f;
+constexpr float POW_EXP_MIN = -87.0f;          // (2^-126 = e^-87.34)
 // 2^-126: what is below it has no reciprocal here.  Heads nearer to
 // saturation count as saturated, a smaller coupling as none.
 constexpr float NORMAL_MIN = 1.17549435e-38f;
@@ -435,27 +436,34 @@ template <int MODEL>
 __device__ __forceinline__ DBase dbase(float psi0, float p1, float p2) {
   DBase B;
   B.psi0 = psi0;
-  B.wet0 = !(psi0 <= -NORMAL_MIN);
-  B.inv_psi0 = B.wet0 ? 0.0f : rcp_a(psi0);
   B.a0 = B.b0 = B.c0 = B.r0 = 0.0f;
   B.m = MODEL == VANGENUCHTEN ? 1.0f - rcp_a(p2) : 0.0f;
+  float lp = 0.0f;               // log of the power of h0 (no number, or -inf, from saturation on)
+  if (MODEL == GARDNER) {
+    B.wet0 = !(psi0 <= -NORMAL_MIN);
+  } else {
+    lp = p2 * log_a(MODEL == HAVERKAMP ? -psi0 : p1 * -psi0);
+    // a power that would be flushed: theta(psi0) is theta_s to below 2^-125
+    // (testing the power itself, after the branch, cost the finest level's
+    // one-colour defect 7%)
+    B.wet0 = !(lp >= POW_EXP_MIN);
+  }
+  B.inv_psi0 = B.wet0 ? 0.0f : rcp_a(psi0);
   if (!B.wet0) {
     if (MODEL == GARDNER) {
       B.a0 = __expf(p1 * psi0);
     } else if (MODEL == HAVERKAMP) {
-      const float lu = fminf(p2 * log_a(-psi0), POW_EXP_MAX);   // h0^beta
+      const float lu = fminf(lp, POW_EXP_MAX);   // h0^beta
       B.a0 = exp_a(lu);
       B.b0 = lu;
       B.r0 = rcp_a(p1 + B.a0);
     } else {
       const float m = B.m;
-      B.a0 = exp_a(fminf(p2 * log_a(p1 * -psi0), POW_EXP_MAX));   // (alpha h0)^n
+      B.a0 = exp_a(fminf(lp, POW_EXP_MAX));   // (alpha h0)^n
       B.b0 = fast_log1p(B.a0);
       B.c0 = exp_a(-m * B.b0);
       B.r0 = rcp_a(1.0f + B.a0);
     }
-    // a flushed power: theta(psi0) is theta_s to below 2^-126
-    if (MODEL != GARDNER) B.wet0 = B.a0 == 0.0f;
   }
   return B;
 }
@@ -569,17 +577,23 @@ __device__ __forceinline__ int feddes_piece(T psi, const Phys<T>& P, T& da) {
   return 3;
 }
 // alpha_F(psi1) - alpha_F(psi0), on pieces k1 and k0.  A correction seldom
-// crosses a kink, so this is a call (by value: a reference would put the
-// physics in memory): inlined, the two ramps at every update cost the served
-// mix 6% (8 requests 8.66 -> 9.16 ms).
-static __device__ __noinline__ float feddes_jump(float psi0, int k0, float psi1, int k1, float h1, float h2, float h3,
-                                                 float h4, float r12, float r34) {
+// crosses a kink, so point updates make it a call (by value: a reference would
+// put the physics in memory): inlined, the two ramps at every update cost the
+// served mix 6% (8 requests 8.66 -> 9.16 ms) and the defect-writing half-sweep
+// of 256^3 6% (125 -> 132 us).  Defects alone, which evaluate it once, take it
+// inline: there the call cost the 256^3 one-colour defect 15% (97 -> 112 us).
+__device__ __forceinline__ float feddes_jump(float psi0, int k0, float psi1, int k1, float h1, float h2, float h3,
+                                             float h4, float r12, float r34) {
   auto value = [=](float psi, int k) {
     if (k == 1) return ramp(h1 - psi, h1 - h2, r12);
     if (k == 3) return ramp(psi - h4, h3 - h4, r34);
     return k == 2 ? 1.0f : 0.0f;
   };
   return value(psi1, k1) - value(psi0, k0);
+}
+static __device__ __noinline__ float feddes_jump_call(float psi0, int k0, float psi1, int k1, float h1, float h2,
+                                                      float h3, float h4, float r12, float r34) {
+  return feddes_jump(psi0, k0, psi1, k1, h1, h2, h3, h4, r12, r34);
 }
 
 // alpha_F in FP64 on a ramp (a call as well: the FP64 operations of both ramps
@@ -600,13 +614,18 @@ __device__ __forceinline__ void sink_direct(double psi, double smax, const Phys<
 }
 
 // S(psi0 + x) - S(psi0), psi0 on piece k0: exact slope * x on a common linear
-// piece.
+// piece.  CALL: the crossing of a kink as a call.
+template <bool CALL>
 __device__ __forceinline__ void sink_delta(float psi0, int k0, float x, float smax, const Phys<float>& P, float& DS,
                                            float& dS) {
   float da;
   const int k1 = feddes_piece(psi0 + x, P, da);
   DS = smax * da * x;
-  if (k1 != k0) DS = smax * feddes_jump(psi0, k0, psi0 + x, k1, P.h1, P.h2, P.h3, P.h4, P.r12, P.r34);
+  if (k1 != k0) {
+    const float j = CALL ? feddes_jump_call(psi0, k0, psi0 + x, k1, P.h1, P.h2, P.h3, P.h4, P.r12, P.r34)
+                         : feddes_jump(psi0, k0, psi0 + x, k1, P.h1, P.h2, P.h3, P.h4, P.r12, P.r34);
+    DS = smax * j;
+  }
   dS = smax * da;
 }
 
@@ -679,8 +698,8 @@ template <>
 __device__ __forceinline__ float tol_of<float>() { return 1e-7f; }
 
 // Storage + sink part at x (the defect's part of N) of cell q of a level, of
-// material m.
-template <typename T, int FORM, int MODEL>
+// material m.  CALL: as for sink_delta.
+template <typename T, int FORM, int MODEL, bool CALL = false>
 __device__ __forceinline__ T storage(const Level<T>& L, T x, T psi0, T p1, T p2, T smax, unsigned m,
                                      const Phys<T>& P) {
   if constexpr (FORM == FORM_DIRECT) {
@@ -693,7 +712,7 @@ __device__ __forceinline__ T storage(const Level<T>& L, T x, T psi0, T p1, T p2,
     return with_law<MODEL>(P, m, [&](auto law, const Phys<T>& Q) {
       float Dth, dth, DS = 0.0f, dS, da0;
       dlaw_fast<decltype(law)::value>(psi0, x, p1, p2, Q, Dth, dth);
-      if (Q.sink && smax > 0.0f) sink_delta(psi0, feddes_piece(psi0, Q, da0), x, smax, Q, DS, dS);
+      if (Q.sink && smax > 0.0f) sink_delta<CALL>(psi0, feddes_piece(psi0, Q, da0), x, smax, Q, DS, dS);
       return Q.a * Dth + DS;
     });
   }
@@ -775,7 +794,7 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
       float Dth, dth;
       dincr<MODEL>(B, x, p1, p2, P, Dth, dth);
       T DS = T(0), dS = T(0);
-      if (has_sink) sink_delta(psi0, sk0, x, smax, P, DS, dS);
+      if (has_sink) sink_delta<true>(psi0, sk0, x, smax, P, DS, dS);
       val = P.a * Dth + DS;
       der = P.a * dth + dS;
     } else {
@@ -954,7 +973,7 @@ __device__ __forceinline__ void cell_sums(const Level<T>& L, const CellOps<T>& c
 // (the expression of apply_N(), so both give the same bits)
 template <typename T, int FORM, int MODEL>
 __device__ __forceinline__ T cell_defect(const Level<T>& L, const Phys<T>& P, const CellOps<T>& c, T dg, T of, T x) {
-  const T val = storage<T, FORM, MODEL>(L, x, c.psi0, c.p1, c.p2, c.smax, c.mat, P);
+  const T val = storage<T, FORM, MODEL, true>(L, x, c.psi0, c.p1, c.p2, c.smax, c.mat, P);
   return c.g - (val + P.xi * x + dg * x - of);
 }
 
