@@ -347,8 +347,7 @@ __device__ void column_solve(const ColArgs& A, int c, float* smem, Level<float>*
           th = theta_only_d<MODEL>(ui, D.p1, D.p2, P64);
           thcur[i] = th;
         }
-        double S, dS;
-        sink_direct(ui, G.smax ? G.smax[i] : 0.0, P64, S, dS);
+        const double S = sink_value(ui, G.smax ? G.smax[i] : 0.0, P64);
         const double di = G.g[i] - ((a * th + S) + (A.xi + db) * ui + flux);
         Ls[0].g[i] = (float)di;
         const_cast<float*>(Ls[0].psi0)[i] = (float)ui;

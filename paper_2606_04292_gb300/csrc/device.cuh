@@ -596,8 +596,12 @@ static __device__ __noinline__ float feddes_jump_call(float psi0, int k0, float 
   return feddes_jump(psi0, k0, psi1, k1, h1, h2, h3, h4, r12, r34);
 }
 
-// alpha_F in FP64 on a ramp (a call as well: the FP64 operations of both ramps
-// would otherwise issue in every update, with or without a sink)
+// alpha_F in FP64: the ramps are calls as well (the FP64 operations of both
+// would otherwise issue in every update, with or without a sink; 257^2 FP64
+// strip +1.3%).  The point solve calls for the one ramp that a psi lies on: a
+// 2000-cell column with root uptake 31.7 ms a step, 35.2 with all of alpha_F in
+// the call, 32.8 with plain products inline (the 777-cell layered column, which
+// has no sink, 9.28, 9.04 and 9.15).  A defect calls for all of it.
 static __device__ __noinline__ double feddes_ramp(double psi, int k, double h1, double h2, double h3, double h4,
                                                   double r12, double r34) {
   return k == 1 ? ramp(h1 - psi, h1 - h2, r12) : ramp(psi - h4, h3 - h4, r34);
@@ -611,6 +615,18 @@ __device__ __forceinline__ void sink_direct(double psi, double smax, const Phys<
   }
   S = a * smax;
   dS = da * smax;
+}
+static __device__ __noinline__ double feddes_alpha(double psi, double h1, double h2, double h3, double h4, double r12,
+                                                   double r34) {
+  Phys<double> P;
+  P.h1 = h1; P.h2 = h2; P.h3 = h3; P.h4 = h4;
+  P.r12 = r12; P.r34 = r34;
+  double da;
+  const int k = feddes_piece(psi, P, da);
+  return k & 1 ? feddes_ramp(psi, k, h1, h2, h3, h4, r12, r34) : (k == 2 ? 1.0 : 0.0);
+}
+__device__ __forceinline__ double sink_value(double psi, double smax, const Phys<double>& P) {
+  return P.sink && smax > 0.0 ? smax * feddes_alpha(psi, P.h1, P.h2, P.h3, P.h4, P.r12, P.r34) : 0.0;
 }
 
 // S(psi0 + x) - S(psi0), psi0 on piece k0: exact slope * x on a common linear
@@ -704,9 +720,7 @@ __device__ __forceinline__ T storage(const Level<T>& L, T x, T psi0, T p1, T p2,
                                      const Phys<T>& P) {
   if constexpr (FORM == FORM_DIRECT) {
     static_assert(sizeof(T) == 8, "direct form is FP64");
-    double S, dS;
-    sink_direct(x, smax, P, S, dS);
-    return P.a * theta_cell<MODEL>(x, p1, p2, m, !L.p1 && !L.p2, P) + S;
+    return P.a * theta_cell<MODEL>(x, p1, p2, m, !L.p1 && !L.p2, P) + sink_value(x, smax, P);
   } else {
     static_assert(sizeof(T) == 4, "increment form is FP32");
     return with_law<MODEL>(P, m, [&](auto law, const Phys<T>& Q) {

@@ -411,8 +411,7 @@ __global__ void __launch_bounds__(256) k_outer_residual64(Level<double> L, Phys<
       th = theta_cell<MODEL>(ui, p1, p2, mat_of<MODEL>(L, i), !L.p1 && !L.p2, P);
       if (th_out) th_out[i] = th;
     }
-    double S, dS;
-    sink_direct(ui, L.smax ? L.smax[i] : 0.0, P, S, dS);
+    const double S = sink_value(ui, L.smax ? L.smax[i] : 0.0, P);
     const double di = L.g[i] - ((P.a * th + S) + (P.xi + db) * ui + flux);
     const unsigned q = pix_of(cs, L.n0, L.n1, L.n2, (unsigned)i, i0, i1, i2);
     r32[q] = (float)di;
@@ -739,8 +738,7 @@ __global__ void __launch_bounds__(256) k_mass_balance64(Level<double> L, Geom G,
       ps = P.lag ? pn : 2.0 * pn - pm;
     }
     const double smax = L.smax ? L.smax[i] : 0.0;
-    double S, dS;
-    sink_direct(psi, smax, P, S, dS);
+    const double S = sink_value(psi, smax, P);
     double cell = (P.a * th1 - hist) + S + P.xi * (psi - ps);
     cell *= V;
     // inflow through this cell's boundary faces (face area A = V / h)
