@@ -596,26 +596,36 @@ static __device__ __noinline__ float feddes_jump_call(float psi0, int k0, float 
   return feddes_jump(psi0, k0, psi1, k1, h1, h2, h3, h4, r12, r34);
 }
 
-// alpha_F in FP64: the ramps are calls as well (the FP64 operations of both
-// would otherwise issue in every update, with or without a sink; 257^2 FP64
-// strip +1.3%).  The point solve calls for the one ramp that a psi lies on: a
-// 2000-cell column with root uptake 31.7 ms a step, 35.2 with all of alpha_F in
-// the call, 32.8 with plain products inline (the 777-cell layered column, which
-// has no sink, 9.28, 9.04 and 9.15).  A defect calls for all of it.
-static __device__ __noinline__ double feddes_ramp(double psi, int k, double h1, double h2, double h3, double h4,
-                                                  double r12, double r34) {
-  return k == 1 ? ramp(h1 - psi, h1 - h2, r12) : ramp(psi - h4, h3 - h4, r34);
+// alpha_F in FP64 on piece k: one ramp, its operands selected (with both
+// inline, their FP64 operations issued in every update, with or without a
+// sink).  CALL: where the physics are known to have a sink only at run time,
+// the ramp is a call: inline, the 257^2 FP64 strip's steps took 1.3% longer;
+// as a call where it is known, the 777-cell layered column's did.
+__device__ __forceinline__ double feddes_ramp(double psi, int k, double h1, double h2, double h3, double h4,
+                                              double r12, double r34) {
+  const bool wet = k == 1;
+  return ramp(wet ? h1 - psi : psi - h4, wet ? h1 - h2 : h3 - h4, wet ? r12 : r34);
 }
+static __device__ __noinline__ double feddes_ramp_call(double psi, int k, double h1, double h2, double h3, double h4,
+                                                       double r12, double r34) {
+  return feddes_ramp(psi, k, h1, h2, h3, h4, r12, r34);
+}
+template <bool CALL>
 __device__ __forceinline__ void sink_direct(double psi, double smax, const Phys<double>& P, double& S, double& dS) {
   double a = 0.0, da = 0.0;
   if (P.sink && smax > 0.0) {
     const int k = feddes_piece(psi, P, da);
     a = k == 2 ? 1.0 : 0.0;
-    if (k & 1) a = feddes_ramp(psi, k, P.h1, P.h2, P.h3, P.h4, P.r12, P.r34);
+    if (k & 1)
+      a = CALL ? feddes_ramp_call(psi, k, P.h1, P.h2, P.h3, P.h4, P.r12, P.r34)
+               : feddes_ramp(psi, k, P.h1, P.h2, P.h3, P.h4, P.r12, P.r34);
   }
   S = a * smax;
   dS = da * smax;
 }
+// S at psi, for a defect: one evaluation a cell, all of it a call (in the point
+// solve that cost a 2000-cell column with root uptake 35.2 ms a step instead of
+// 31.7; 32.7 with plain products inline)
 static __device__ __noinline__ double feddes_alpha(double psi, double h1, double h2, double h3, double h4, double r12,
                                                    double r34) {
   Phys<double> P;
@@ -815,7 +825,7 @@ __device__ __forceinline__ T point_solve(T cc, T f, T x0, T psi0, T p1, T p2, T 
       T th, dth, S, dS;
       law.eval(x, P, th, dth);
       S = dS = T(0);
-      if (SINK != 0) sink_direct(x, smax, P, S, dS);
+      if (SINK != 0) sink_direct<(SINK < 0)>(x, smax, P, S, dS);
       val = P.a * th + S;
       der = P.a * dth + dS;
     }
