@@ -50,12 +50,12 @@ DTYPE = {2: "f32 inner / f64 outer, f64 state", 1: "f32 inner / float-float (f32
 # 256^3 (8,388,608 cells, colour-split parameters, 128-thread blocks, two
 # planes), from an ncu capture of this kernel (dram__bytes_read.sum +
 # dram__bytes_write.sum); the roofline's traffic.
-TRAFFIC_PER_LAUNCH = {("sweep32", 8388608): 318.5e6}
+TRAFFIC_PER_LAUNCH = {("sweep32", 8388608): 318.8e6}
 # What binds that launch instead of DRAM, from the same capture: the share of
 # issue slots active (smsp__issue_active) and of DRAM bandwidth in use.
-BINDING_PER_LAUNCH = {("sweep32", 8388608): {"limit": "instruction issue", "issue_active": 0.81,
-                                             "dram_throughput": 0.42, "thread_instructions_per_update": 345,
-                                             "source": "ncu --set full (profiles/sweep32_drainage256_mixed.md)"}}
+BINDING_PER_LAUNCH = {("sweep32", 8388608): {"limit": "instruction issue", "issue_active": 0.80,
+                                             "dram_throughput": 0.50, "thread_instructions_per_update": 292,
+                                             "source": "ncu (profiles/sweep32_drainage256_mixed.md)"}}
 
 BYTES_PER_CELL = {
     "sweep32": 28.0,
