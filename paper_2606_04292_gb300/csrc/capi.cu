@@ -1421,7 +1421,7 @@ void batch_tail(richards_batcher* b, std::vector<BatchCtx>& B, const std::vector
   const richards_opts& o = B[who[0]].c->opts;
   for (size_t a = 0; a < who.size(); a += rich::BATCH_MAX) {
     rich::BList list{};
-    int blocks = 1;                   // (one size a launch: the biggest level's)
+    int blocks = 1;                   // (one size a launch: at most what the biggest level takes)
     for (size_t q = a; q < who.size() && q < a + rich::BATCH_MAX; ++q) {
       list.job[list.n++] = B[who[q]].slot * MAXLEV + l;
       blocks = std::max(blocks, tail_shape<float>(B[who[q]].c, l).blocks);

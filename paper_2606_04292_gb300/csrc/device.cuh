@@ -444,8 +444,6 @@ __device__ __forceinline__ DBase dbase(float psi0, float p1, float p2) {
   } else {
     lp = p2 * log_a(MODEL == HAVERKAMP ? -psi0 : p1 * -psi0);
     // a power that would be flushed: theta(psi0) is theta_s to below 2^-125
-    // (testing the power itself, after the branch, cost the finest level's
-    // one-colour defect 7%)
     B.wet0 = !(lp >= POW_EXP_MIN);
   }
   B.inv_psi0 = B.wet0 ? 0.0f : rcp_a(psi0);
